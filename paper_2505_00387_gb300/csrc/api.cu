@@ -748,15 +748,30 @@ int aahrt_apply_stage(aahrt_plan *plan, int stage, const void *in, void *out, vo
     float *fo = static_cast<float *>(out);
     float2 *co = static_cast<float2 *>(out);
     switch (stage) {
-        case 0: e = launch_r2c(p, true, fi, co, st); break;
-        case 1: e = launch_slice(p, false, ci, co, st); break;
-        case 2: e = launch_c2r(p, false, ci, fo, EPI_STORE, nullptr, FistaArgs{}, st); break;
-        case 3: e = launch_r2c(p, false, fi, co, st); break;
-        case 4:
-            e = launch_ybound(p, ci, st);
-            if (!e) e = launch_slice(p, true, ci, co, st);
+        case 0: e = launch_r2c(p, true, fi, co, st, false, true); break;
+        case 2:
+            e = launch_c2r(p, false, ci, fo, EPI_STORE, nullptr, FistaArgs{}, st, false, true);
             break;
-        case 5: e = launch_c2r(p, true, ci, fo, EPI_STORE, nullptr, FistaArgs{}, st); break;
+        case 3: e = launch_r2c(p, false, fi, co, st, false, true); break;
+        case 1:
+        case 4: {
+            const bool adj = stage == 4;
+            e = adj ? launch_ybound(p, ci, st) : cudaSuccess;
+            if (e) break;
+            if (!p.bins_fastest) {
+                e = launch_slice(p, adj, ci, co, st);
+                break;
+            }
+            // through the workspace, which holds the plan's own layout
+            float2 *src = adj ? p.Y : p.X, *dst = adj ? p.X : p.Y;
+            e = launch_transpose_spec(p, !adj, ci, src, true, st);
+            if (!e) e = launch_slice(p, adj, src, dst, st);
+            if (!e) e = launch_transpose_spec(p, adj, dst, co, false, st);
+            break;
+        }
+        case 5:
+            e = launch_c2r(p, true, ci, fo, EPI_STORE, nullptr, FistaArgs{}, st, false, true);
+            break;
         default: return set_error(AAHRT_ERR_INVALID_ARG, "stage must be 0..5");
     }
     return e ? cuda_fail(e, "stage launch") : AAHRT_OK;

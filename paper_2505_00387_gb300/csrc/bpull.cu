@@ -16,9 +16,8 @@ namespace aahrt {
 
 struct PullArgs {
     const float2 *__restrict__ D;       // data spectrum [k][ntr]
-    const SliceGroup *__restrict__ groups;
     const float2 *__restrict__ tw;
-    int nbins, nq, ntheta, nos, Lq, cq, ngroup;
+    int nbins, nq, ntheta, nos, Lq, cq, ngroup, tgroup;
     int nx, ny;
     float x0, dx, y0, dy, r2max;
     double inv_nos_dq;      // 1 / (nos dq): wavenumber of grid step u
@@ -55,7 +54,7 @@ pull_kernel(const PullArgs a, float2 *__restrict__ X) {
     float *smf = reinterpret_cast<float *>(smem_f4);
     const int gi = blockIdx.x % a.ngroup;
     const int k = blockIdx.x / a.ngroup;
-    const SliceGroup g = a.groups[gi];
+    struct { int ja, nj; } g{gi * a.tgroup, min(a.tgroup, a.ntheta - gi * a.tgroup)};
     const int lds = ld_split(a.nos);
     const int mask = a.nos - 1;
     float *Gre = smf, *Gim = smf + g.nj * lds;
@@ -140,14 +139,13 @@ extern "C" int aahrt_velocity_scan_grid(aahrt_plan *plan, const aahrt_grid *grid
         max_smem = mx - (int)at.sharedSizeBytes;
     }
     // one group's split q grid (re and im planes of every owned slice)
-    const size_t smem = (size_t)p.tgroup * ld_split(p.nos) * 2 * sizeof(float);
+    const size_t smem = (size_t)p.pull_group * ld_split(p.nos) * 2 * sizeof(float);
     if ((int)smem > max_smem)
         return set_error(AAHRT_ERR_UNSUPPORTED, "the grid scan's q grids (%zu bytes) exceed "
                          "shared memory; lower theta_group", smem);
     if ((e = launch_stretch_data(p, d, p.Y, st))) return cuda_fail(e, "stretch+FFT launch");
     PullArgs a;
     a.D = p.Y;
-    a.groups = p.groups;
     a.tw = p.tw_q;
     a.nbins = p.nbins;
     a.nq = p.nq;
@@ -155,7 +153,8 @@ extern "C" int aahrt_velocity_scan_grid(aahrt_plan *plan, const aahrt_grid *grid
     a.nos = p.nos;
     a.Lq = p.Lq;
     a.cq = p.cq;
-    a.ngroup = p.ngroup;
+    a.tgroup = p.pull_group;
+    a.ngroup = (p.ntheta + p.pull_group - 1) / p.pull_group;
     a.nx = grid->nx;
     a.ny = grid->ny;
     a.x0 = (float)grid->x0;
@@ -170,7 +169,7 @@ extern "C" int aahrt_velocity_scan_grid(aahrt_plan *plan, const aahrt_grid *grid
     a.kscale = 1.0 / (p.nfft * p.ds);
     a.scale = (float)(1.0 / p.nfft);
     prof_begin(p, 4, st);
-    pull_kernel<<<p.nbins * p.ngroup, 256, smem, st>>>(a, p.X);
+    pull_kernel<<<p.nbins * a.ngroup, 256, smem, st>>>(a, p.X);
     prof_end(p, st);
     p.launches[4]++;
     if ((e = cudaGetLastError())) return cuda_fail(e, "pull launch");

@@ -60,11 +60,19 @@ struct PnBlock {
     int rep;
 };
 
+// One cube's spectrum block for the transposition between the two spectrum
+// layouts: ncol columns of nbins complex values from complex offset off.
+struct SpecBlock {
+    long long off;
+    int ncol;
+};
+
 // Column group of the time-axis kernels (at most 2*pairs columns).
 struct ColGroup {
     long long real_off;  // float offset of the group's first column in the
                          // real (time-domain) array, row 0
     long long spec_off;  // complex offset of its first column in the spectrum
+    long long bins_off;  // the same in a bins-fastest spectrum [column][bin]
     int ld_real, ld_spec;  // row strides (elements)
     int ncol;
     int cube;            // cube (or gather) the columns belong to
@@ -124,6 +132,14 @@ struct Plan {
     // q spreading
     int nos = 0, Lq = 0, cq = 0;
     double beta = 0;
+    // Spectra X[q][theta][bin], Y[trace][bin] per cube (slice_tiles.cuh)
+    // instead of X[bin][q][theta], Y[bin][trace]; tile = bins per block tile.
+    bool bins_fastest = false;
+    int tile = 0;
+    double phicap = 0;             // bound on one kernel weight
+    SpecBlock *spec_model = nullptr, *spec_data = nullptr;   // every cube's spectrum block
+    int max_ntr = 0;               // largest fold
+    int pull_group = 0;            // azimuth slices per block of the pull scan
     int tgroup = 0, ngroup = 1;   // slices per group, groups per cube
     long long model_len = 0, data_len = 0, cols_model = 0;
     // device tables
@@ -233,14 +249,22 @@ inline cudaError_t raise_smem_limit(F *func, int max_smem) {
 int set_error(int code, const char *fmt, ...);
 int cuda_fail(cudaError_t e, const char *what);
 
-// stage launchers (stream-ordered, no synchronisation)
+// stage launchers (stream-ordered, no synchronisation); `natural`: the
+// spectrum is X[bin][q][theta] / Y[bin][trace] whatever the plan's layout
 cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
-                       cudaStream_t st, bool blocked = false);
+                       cudaStream_t st, bool blocked = false, bool natural = false);
 cudaError_t launch_c2r(Plan &p, bool model_side, const float2 *in, float *out,
                        int epi, const float *aux, FistaArgs fa, cudaStream_t st,
-                       bool blocked = false);
+                       bool blocked = false, bool natural = false);
 cudaError_t launch_slice(Plan &p, bool adjoint, const float2 *in, float2 *out,
                          cudaStream_t st, int *counter = nullptr);
+// the slice step of bins-fastest spectra (slice_tiles.cuh)
+cudaError_t launch_slice_tiles(Plan &p, bool adjoint, const float2 *in, float2 *out,
+                               cudaStream_t st, int *counter);
+cudaError_t configure_tile_kernels(Plan &p, int num_sms, int max_smem);
+// a spectrum between its natural and its bins-fastest layout (every cube)
+cudaError_t launch_transpose_spec(Plan &p, bool model_side, const float2 *in, float2 *out,
+                                  bool to_bins, cudaStream_t st);
 // fused synthesis + analysis of one FISTA half-iteration (column-blocked state)
 cudaError_t launch_c2r_r2c(Plan &p, bool model_side, float2 *spec, const float *aux,
                            FistaArgs fa, cudaStream_t st);

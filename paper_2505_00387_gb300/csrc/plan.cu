@@ -202,7 +202,7 @@ void free_plan(Plan *p) {
                     p->stage_m, p->stage_d, p->zb, p->mb, p->rb, p->db, p->vjp_ws,
                     p->cube_gt, p->cube_acc, p->dseg, p->tc_tiles, p->wav, p->wtmp,
                     p->qn, p->qv, p->pn_blk, p->pn_rho, p->pn_c, p->ymax, p->wsum,
-                    p->geo_adj};
+                    p->geo_adj, p->spec_model, p->spec_data};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     cudaSetDevice(cur);
@@ -228,6 +228,31 @@ static int validate_geom(const aahrt_geom *g, int idx, bool q_explicit) {
         if (!std::isfinite(g->hx[h]) || !std::isfinite(g->hy[h]))
             return set_error(AAHRT_ERR_NONFINITE, "geometry %d: offset %d not finite", idx, h);
     return AAHRT_OK;
+}
+
+// Bins per tile and azimuth slices per work item of the bins-fastest slice
+// kernels.  An item walks its nj slices and one more (the neighbour its first
+// or last interval shares), so its time goes as (nj + 1) x tile, and the items
+// run in ceil(items / resident blocks) rounds: the pair with the smallest
+// product, larger tiles (a whole warp on one trace) on a tie.
+static void choose_tiles(Plan &p, bool group_fixed, int ncube, int sms) {
+    const long long blocks = (long long)sms * (p.nos == 512 ? 1 : 3);
+    double best = 1e300;
+    const int given = p.tgroup;
+    for (int tile = p.nos <= 128 ? 32 : 16; tile >= 16; tile /= 2)
+        for (int ng = 1; ng <= p.ntheta; ++ng) {
+            const int nj = group_fixed ? given : (p.ntheta + ng - 1) / ng;
+            const long long groups = (p.ntheta + nj - 1) / nj;
+            const long long items = groups * ((p.nbins + tile - 1) / tile) * ncube;
+            const double rounds = items > blocks ? (double)items / blocks + 0.5 : 1.0;
+            const double cost = rounds * (nj + 1) * tile * (tile == 16 && p.nos <= 128 ? 1.15 : 1.0);
+            if (cost < best) {
+                best = cost;
+                p.tile = tile;
+                p.tgroup = nj;
+            }
+            if (group_fixed) break;
+        }
 }
 
 // Build a plan for ncube cubes.  geoms has ndist entries: ndist == ncube
@@ -428,6 +453,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
                          : (float)(1.0 / es_fourier((double)(l - p->cq) / p->nos, p->beta, W));
 
     // --------------------------------------------------- azimuth groups
+    p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512;
     const size_t per_slice = (size_t)std::max(ld_interleaved(p->nos), ld_split(p->nos)) *
                              sizeof(float2);
     if (opts.theta_group > 0) {
@@ -452,6 +478,19 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         }
     }
     if (p->tgroup > kMaxGroupSlices) p->tgroup = kMaxGroupSlices;
+    p->pull_group = p->tgroup;
+    if (p->bins_fastest) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+        choose_tiles(*p, opts.theta_group > 0, ncube, sms);
+        // a column's bins are contiguous, so fewer pairs per time block cost no
+        // bandwidth: as few as it takes to give every SM a block on either side
+        long long ntr = 0;
+        for (int c = 0; c < ncube; ++c) ntr += geoms[ndist == 1 ? 0 : c].ntr;
+        const long long cols = std::min<long long>(ntr, (long long)ncube * p->nq * p->ntheta);
+        while (opts.time_pairs == 0 && p->pairs > 1 && cols / (2 * p->pairs) < sms) p->pairs /= 2;
+        p->lp = ilog2(p->pairs);
+    }
     p->ngroup = (p->ntheta + p->tgroup - 1) / p->tgroup;
     if (p->ngroup == 1) p->tgroup = p->ntheta;
 
@@ -532,7 +571,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
             for (int j = 0; j < J; ++j)
                 for (int g0 = 0; g0 < G; g0 += cpg)
                     cgm.push_back(ColGroup{((long long)l * J + j) * G + g0,
-                                           ((long long)j * nb * nq + l) * G + g0,
+                                           ((long long)j * nb * nq + l) * G + g0, 0,
                                            (int)(C * G), nq * G, std::min(cpg, G - g0), 0});
         const CubeGeo &cg0 = cg[0];
         std::vector<int> rank(p->ntr[0]), slice(p->ntr[0]);
@@ -546,7 +585,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
             const int cnt = cg0.start[j + 1] - cg0.start[j];
             for (int g0 = 0; g0 < G; g0 += cpg)
                 cgd.push_back(ColGroup{(long long)h * G + g0,
-                                       (nb * cg0.start[j] + rank[h]) * G + g0,
+                                       (nb * cg0.start[j] + rank[h]) * G + g0, 0,
                                        p->ntr[0] * G, cnt * G, std::min(cpg, G - g0), 0});
         }
     }
@@ -555,6 +594,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
             ColGroup q;
             q.real_off = (long long)c * p->ntau * C + c0;
             q.spec_off = (long long)c * p->nbins * C + c0;
+            q.bins_off = ((long long)c * C + c0) * p->nbins;
             q.ld_real = (int)C;
             q.ld_spec = (int)C;
             q.ncol = (int)std::min<long long>(cpg, C - c0);
@@ -566,6 +606,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
             ColGroup q;
             q.real_off = p->data_off[c] + h0;
             q.spec_off = y_off[c] + h0;
+            q.bins_off = y_off[c] + (long long)h0 * p->nbins;
             q.ld_real = p->ntr[c];
             q.ld_spec = p->ntr[c];
             q.ncol = std::min(cpg, p->ntr[c] - h0);
@@ -608,8 +649,8 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     } else {
         fit_es_poly(W, p->beta, &p->poly);
     }
-    {   // bound on the summed kernel weights of one trace, with margin
-        double mx = 0.0;
+    {   // bounds on the summed and on the single kernel weights of one trace, with margin
+        double mx = 0.0, one = 0.0;
         for (int s = 0; s <= 2000; ++s) {
             const double g = -0.5 + s / 2000.0;
             double sum = 0.0;
@@ -617,10 +658,12 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
                 double v = 0.0;
                 for (int d = W + 1; d >= 0; --d) v = v * g + p->poly.c[d][i];
                 sum += std::fabs(v);
+                one = std::max(one, std::fabs(v));
             }
             mx = std::max(mx, sum);
         }
         p->phimax = 1.05 * mx;
+        p->phicap = 1.001 * one;
     }
 
     // ------------------------------------------------------- twiddles
@@ -710,6 +753,16 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         AAHRT_TRY(upload(&p->pn_rho, rho), "upload offsets");
         AAHRT_TRY(cudaMalloc((void **)&p->pn_c, rho.size() * sizeof(float2)), "alloc offsets");
     }
+    if (p->bins_fastest) {
+        std::vector<SpecBlock> bm, bd;
+        for (int c = 0; c < ncube; ++c) {
+            bm.push_back(SpecBlock{(long long)c * p->nbins * C, (int)C});
+            bd.push_back(SpecBlock{y_off[c], p->ntr[c]});
+            p->max_ntr = std::max(p->max_ntr, p->ntr[c]);
+        }
+        AAHRT_TRY(upload(&p->spec_model, bm), "upload spectrum blocks");
+        AAHRT_TRY(upload(&p->spec_data, bd), "upload spectrum blocks");
+    }
     AAHRT_TRY(cudaMalloc((void **)&p->counters, 16 * sizeof(int)), "alloc counters");
     AAHRT_TRY(cudaMemset(p->counters, 0, 16 * sizeof(int)), "clear counters");
     p->S = DevResampler{p->posS, nullptr, p->ns, p->ns};
@@ -743,9 +796,12 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         p->smem_sfwd = direct_smem_fwd(p->tgroup, p->ngroup > 1 ? 1 : 0, p->nq);
         p->smem_sadj = direct_smem_adj(p->tgroup, p->nq, p->direct_chunk);
     } else {
-        p->smem_sfwd = (size_t)(p->tgroup + (p->ngroup > 1 ? 1 : 0)) * ld_interleaved(p->nos) *
+        // (the bins-fastest kernels need less: a requested group is held to
+        // the same limit whichever kernel serves it)
+        const int tg = p->bins_fastest ? p->pull_group : p->tgroup;
+        p->smem_sfwd = (size_t)(tg + (tg < p->ntheta ? 1 : 0)) * ld_interleaved(p->nos) *
                        sizeof(float2);
-        p->smem_sadj = (size_t)p->tgroup * ld_split(p->nos) * 2 * sizeof(float);
+        p->smem_sadj = (size_t)tg * ld_split(p->nos) * 2 * sizeof(float);
     }
     int max_smem = 0;
     AAHRT_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin,
@@ -777,6 +833,8 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         AAHRT_TRY(configure_tc_kernels(*p, num_sms, max_smem), "tensor-core kernel configuration");
     } else if (direct) {
         AAHRT_TRY(configure_direct_kernels(*p, num_sms, max_smem), "direct kernel configuration");
+    } else if (p->bins_fastest) {
+        AAHRT_TRY(configure_tile_kernels(*p, num_sms, max_smem), "slice kernel configuration");
     } else {
         AAHRT_TRY(configure_slice_kernels(*p, num_sms, max_smem), "slice kernel configuration");
     }

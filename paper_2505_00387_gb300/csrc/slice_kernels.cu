@@ -1,5 +1,8 @@
 // Fourier slice stage of the AAHRT (Algorithm 1 step 3 and its exact
-// transpose; eqs. Inv_op, inv_GFST and the theta factors of eq. thli).
+// transpose; eqs. Inv_op, inv_GFST and the theta factors of eq. thli), one
+// bin per work item on natural-order spectra X[bin][q][theta], Y[bin][trace]:
+// the plans whose q grid (16 points, or more than 512) the bins-fastest
+// kernels of slice_tiles.cuh do not serve.
 //
 // Forward, per bin k and trace h (scale = 1/Nfft folds the synthesis factor):
 //   Y[k][h] = scale * sum_{s=0,1} w_s(h) * sum_l X[k][l][j_s(h)] exp(-2 pi i f_k q_l r_h^2)
@@ -428,6 +431,13 @@ cudaError_t launch_slice(Plan &p, bool adjoint, const float2 *in, float2 *out,
         prof_begin(p, stage, st);
         e = p.precision == 1 ? launch_slice_tc(p, adjoint, in, out, st, ctr)
                              : launch_slice_direct(p, adjoint, in, out, st, ctr);
+        prof_end(p, st);
+        p.launches[stage]++;
+        return e;
+    }
+    if (p.bins_fastest) {
+        prof_begin(p, stage, st);
+        e = launch_slice_tiles(p, adjoint, in, out, st, ctr);
         prof_end(p, st);
         p.launches[stage]++;
         return e;
