@@ -135,8 +135,10 @@ typedef struct {
     double fmax;        /* highest kept stretched frequency in 1/s^2; 0 = all */
     int time_pairs;     /* column pairs per time-kernel block (1, 2, 4 or 8);
                            0 = automatic (8192 / Nfft clamped to [2, 8] up to
-                           Nfft = 8192, 1 beyond; fewer for plans of few
-                           columns, down to a block per SM) */
+                           Nfft = 8192, 1 beyond).  Plans whose time stages
+                           hold the FFT in registers (Nfft 512..8192 with a
+                           spreading kernel on 32..512 q points) use it for
+                           aahrt_apply_stage and the pull scan only */
     int autotune;       /* 1: pick spread_width, theta_group and time_pairs
                            at plan creation (see aahrt_plan_create); fields
                            set explicitly above are kept */

@@ -205,10 +205,11 @@ __global__ void reblock_kernel(const float *__restrict__ src, float *__restrict_
 
 static cudaError_t reblock(Plan &p, bool model_side, const float *src, float *dst,
                            bool to_blocked, cudaStream_t st) {
-    const int n = model_side ? p.ncg_model : p.ncg_data;
-    reblock_kernel<<<n, 256, 0, st>>>(src, dst, model_side ? p.cg_model : p.cg_data,
-                                      model_side ? p.cg_model_blk : p.cg_data_blk,
-                                      model_side ? p.ntau : p.nt, p.lp + 1,
+    const int n = model_side ? p.ncg_model_blk : p.ncg_data_blk;
+    const ColGroup *nat = p.bins_fastest ? (model_side ? p.cg_model_pair : p.cg_data_pair)
+                                         : (model_side ? p.cg_model : p.cg_data);
+    reblock_kernel<<<n, 256, 0, st>>>(src, dst, nat, model_side ? p.cg_model_blk : p.cg_data_blk,
+                                      model_side ? p.ntau : p.nt, p.blk_lp + 1,
                                       to_blocked ? 1 : 0);
     p.launches[6]++;
     return cudaGetLastError();
@@ -330,7 +331,8 @@ static int run_iterations(Plan &p, int iters, float gamma, float thresh,
                           const std::vector<double> &betas, const float2 *cube_gt,
                           cudaStream_t st) {
     cudaError_t e;
-    if (p.nw == 0 && p.smem_fused_model > 0 && p.smem_fused_data > 0 && iters > 0) {
+    if (p.nw == 0 && iters > 0 &&
+        (p.bins_fastest || (p.smem_fused_model > 0 && p.smem_fused_data > 0))) {
         // Fused half-iterations: the stretch+FFT of z runs once up front, then
         // per iteration slice -> (synthesis + residual + U^T FFT) -> slice^T
         // -> (synthesis + update + stretch+FFT of the new z).  The same

@@ -161,10 +161,19 @@ struct Plan {
     long long slice_items = 0;
     int *counters = nullptr;       // work counters of the persistent kernels
     ColGroup *cg_model = nullptr, *cg_data = nullptr;
-    // the same column groups over column-blocked arrays [group][row][2*pairs]
-    // (the solver's internal state), every group's rows one contiguous slab
+    // column groups over column-blocked arrays [group][row][2*pairs] (the
+    // solver's internal state), every group's rows one contiguous slab
     ColGroup *cg_model_blk = nullptr, *cg_data_blk = nullptr;
     int ncg_model = 0, ncg_data = 0;
+    // the row-major column groups with the columns of the blocked ones (2 per
+    // group in bins-fastest plans, whose time kernels own a pair; else the
+    // groups above), and the blocked groups' number and log2(pairs)
+    ColGroup *cg_model_pair = nullptr, *cg_data_pair = nullptr;
+    int ncg_model_blk = 0, ncg_data_blk = 0, blk_lp = 0;
+    int frame_pairs = 0;           // column pairs per register-FFT block
+    int frame_ahead = 0;           // such blocks resident on the device
+    float *frac_s = nullptr, *frac_u = nullptr;   // the resamplers' fractions alone
+    int sc_i0 = 0, sc_n0 = 0;      // U^T: rows scattered from sc_i0, gathered below sc_n0
     long long mblk_len = 0, dblk_len = 0;
     RowPos *posS = nullptr, *posU = nullptr;       // resampler tables
     RowRange *rngST = nullptr, *rngUT = nullptr;
@@ -262,6 +271,13 @@ cudaError_t launch_slice(Plan &p, bool adjoint, const float2 *in, float2 *out,
 cudaError_t launch_slice_tiles(Plan &p, bool adjoint, const float2 *in, float2 *out,
                                cudaStream_t st, int *counter);
 cudaError_t configure_tile_kernels(Plan &p, int num_sms, int max_smem);
+// the time stages of bins-fastest spectra (time_fft.cuh): op 0 analysis,
+// 1 synthesis, 2 both fused; bound: raise the plan's spectrum bound table
+bool frame_serves(int L, int nt, int ntau, int ns, int max_smem);
+cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem);
+cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *in, void *out,
+                         const float *aux, const FistaArgs &fa, bool blocked, bool bound,
+                         cudaStream_t st);
 // a spectrum between its natural and its bins-fastest layout (every cube)
 cudaError_t launch_transpose_spec(Plan &p, bool model_side, const float2 *in, float2 *out,
                                   bool to_bins, cudaStream_t st);

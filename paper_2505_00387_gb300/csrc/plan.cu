@@ -202,7 +202,8 @@ void free_plan(Plan *p) {
                     p->stage_m, p->stage_d, p->zb, p->mb, p->rb, p->db, p->vjp_ws,
                     p->cube_gt, p->cube_acc, p->dseg, p->tc_tiles, p->wav, p->wtmp,
                     p->qn, p->qv, p->pn_blk, p->pn_rho, p->pn_c, p->ymax, p->wsum,
-                    p->geo_adj, p->spec_model, p->spec_data};
+                    p->geo_adj, p->spec_model, p->spec_data,
+                    p->cg_model_pair, p->cg_data_pair, p->frac_s, p->frac_u};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     cudaSetDevice(cur);
@@ -453,7 +454,10 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
                          : (float)(1.0 / es_fourier((double)(l - p->cq) / p->nos, p->beta, W));
 
     // --------------------------------------------------- azimuth groups
-    p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512;
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
+    p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512 &&
+                      frame_serves(p->L, p->nt, p->ntau, p->ns, optin);
     const size_t per_slice = (size_t)std::max(ld_interleaved(p->nos), ld_split(p->nos)) *
                              sizeof(float2);
     if (opts.theta_group > 0) {
@@ -483,13 +487,6 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
         choose_tiles(*p, opts.theta_group > 0, ncube, sms);
-        // a column's bins are contiguous, so fewer pairs per time block cost no
-        // bandwidth: as few as it takes to give every SM a block on either side
-        long long ntr = 0;
-        for (int c = 0; c < ncube; ++c) ntr += geoms[ndist == 1 ? 0 : c].ntr;
-        const long long cols = std::min<long long>(ntr, (long long)ncube * p->nq * p->ntheta);
-        while (opts.time_pairs == 0 && p->pairs > 1 && cols / (2 * p->pairs) < sms) p->pairs /= 2;
-        p->lp = ilog2(p->pairs);
     }
     p->ngroup = (p->ntheta + p->tgroup - 1) / p->tgroup;
     if (p->ngroup == 1) p->tgroup = p->ntheta;
@@ -589,43 +586,54 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
                                        p->ntr[0] * G, cnt * G, std::min(cpg, G - g0), 0});
         }
     }
-    for (int c = 0; c < (tc ? 0 : ncube); ++c)
-        for (long long c0 = 0; c0 < C; c0 += cpg) {
-            ColGroup q;
-            q.real_off = (long long)c * p->ntau * C + c0;
-            q.spec_off = (long long)c * p->nbins * C + c0;
-            q.bins_off = ((long long)c * C + c0) * p->nbins;
-            q.ld_real = (int)C;
-            q.ld_spec = (int)C;
-            q.ncol = (int)std::min<long long>(cpg, C - c0);
-            q.cube = c;
-            cgm.push_back(q);
-        }
-    for (int c = 0; c < (tc ? 0 : ncube); ++c)
-        for (int h0 = 0; h0 < p->ntr[c]; h0 += cpg) {
-            ColGroup q;
-            q.real_off = p->data_off[c] + h0;
-            q.spec_off = y_off[c] + h0;
-            q.bins_off = y_off[c] + (long long)h0 * p->nbins;
-            q.ld_real = p->ntr[c];
-            q.ld_spec = p->ntr[c];
-            q.ncol = std::min(cpg, p->ntr[c] - h0);
-            q.cube = c;
-            cgd.push_back(q);
-        }
+    auto column_groups = [&](int cols, std::vector<ColGroup> *m, std::vector<ColGroup> *d) {
+        for (int c = 0; c < ncube; ++c)
+            for (long long c0 = 0; c0 < C; c0 += cols) {
+                ColGroup q;
+                q.real_off = (long long)c * p->ntau * C + c0;
+                q.spec_off = (long long)c * p->nbins * C + c0;
+                q.bins_off = ((long long)c * C + c0) * p->nbins;
+                q.ld_real = (int)C;
+                q.ld_spec = (int)C;
+                q.ncol = (int)std::min<long long>(cols, C - c0);
+                q.cube = c;
+                m->push_back(q);
+            }
+        for (int c = 0; c < ncube; ++c)
+            for (int h0 = 0; h0 < p->ntr[c]; h0 += cols) {
+                ColGroup q;
+                q.real_off = p->data_off[c] + h0;
+                q.spec_off = y_off[c] + h0;
+                q.bins_off = y_off[c] + (long long)h0 * p->nbins;
+                q.ld_real = p->ntr[c];
+                q.ld_spec = p->ntr[c];
+                q.ncol = std::min(cols, p->ntr[c] - h0);
+                q.cube = c;
+                d->push_back(q);
+            }
+    };
+    if (!tc) column_groups(cpg, &cgm, &cgd);
     p->ncg_model = (int)cgm.size();
     p->ncg_data = (int)cgd.size();
-    std::vector<ColGroup> cgmb = cgm, cgdb = cgd;
+    // the solver's blocked state: the same groups, or single pairs where the
+    // register-FFT kernels run it
+    const int bcols = p->bins_fastest ? 2 : cpg;
+    std::vector<ColGroup> cgmp, cgdp;
+    if (p->bins_fastest) column_groups(2, &cgmp, &cgdp);
+    std::vector<ColGroup> cgmb = p->bins_fastest ? cgmp : cgm, cgdb = p->bins_fastest ? cgdp : cgd;
+    p->blk_lp = p->bins_fastest ? 0 : p->lp;
+    p->ncg_model_blk = (int)cgmb.size();
+    p->ncg_data_blk = (int)cgdb.size();
     for (size_t gi = 0; gi < cgmb.size(); ++gi) {
-        cgmb[gi].real_off = (long long)gi * p->ntau * cpg;
-        cgmb[gi].ld_real = cpg;
+        cgmb[gi].real_off = (long long)gi * p->ntau * bcols;
+        cgmb[gi].ld_real = bcols;
     }
     for (size_t gi = 0; gi < cgdb.size(); ++gi) {
-        cgdb[gi].real_off = (long long)gi * p->nt * cpg;
-        cgdb[gi].ld_real = cpg;
+        cgdb[gi].real_off = (long long)gi * p->nt * bcols;
+        cgdb[gi].ld_real = bcols;
     }
-    p->mblk_len = (long long)p->ncg_model * p->ntau * cpg;
-    p->dblk_len = (long long)p->ncg_data * p->nt * cpg;
+    p->mblk_len = (long long)p->ncg_model_blk * p->ntau * bcols;
+    p->dblk_len = (long long)p->ncg_data_blk * p->nt * bcols;
 
     // ------------------------------------------------------ resamplers
     std::vector<double> upos(p->ns), vpos(p->nt);
@@ -721,6 +729,23 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     }
     AAHRT_TRY(upload(&p->cg_model, cgm), "upload column groups");
     AAHRT_TRY(upload(&p->cg_data, cgd), "upload column groups");
+    if (p->bins_fastest) {
+        AAHRT_TRY(upload(&p->cg_model_pair, cgmp), "upload column groups");
+        AAHRT_TRY(upload(&p->cg_data_pair, cgdp), "upload column groups");
+        auto fractions = [](const std::vector<RowPos> &pos) {     // whole float4s
+            std::vector<float> f((pos.size() + 3) / 4 * 4, 0.f);
+            for (size_t i = 0; i < pos.size(); ++i) f[i] = pos[i].fr;
+            return f;
+        };
+        AAHRT_TRY(upload(&p->frac_s, fractions(posS)), "upload resamplers");
+        AAHRT_TRY(upload(&p->frac_u, fractions(posU)), "upload resamplers");
+        // from row sc_i0 on every data row starts at a new frame row; the rows
+        // before it reach frame rows below sc_n0
+        p->sc_i0 = p->nt - 1;
+        while (p->sc_i0 > 0 && posU[p->sc_i0 - 1].fl < posU[p->sc_i0].fl) --p->sc_i0;
+        const int reach = p->interp == AAHRT_INTERP_KEYS ? 2 : 1;
+        p->sc_n0 = p->sc_i0 > 0 ? std::min(p->ns, posU[p->sc_i0 - 1].fl + reach + 1) : 0;
+    }
     AAHRT_TRY(upload(&p->cg_model_blk, cgmb), "upload column groups");
     AAHRT_TRY(upload(&p->cg_data_blk, cgdb), "upload column groups");
     AAHRT_TRY(upload(&p->posS, posS), "upload resamplers");
@@ -835,6 +860,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         AAHRT_TRY(configure_direct_kernels(*p, num_sms, max_smem), "direct kernel configuration");
     } else if (p->bins_fastest) {
         AAHRT_TRY(configure_tile_kernels(*p, num_sms, max_smem), "slice kernel configuration");
+        AAHRT_TRY(configure_frame_kernels(*p, num_sms, max_smem), "time kernel configuration");
     } else {
         AAHRT_TRY(configure_slice_kernels(*p, num_sms, max_smem), "slice kernel configuration");
     }

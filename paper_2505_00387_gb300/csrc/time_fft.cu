@@ -1,0 +1,85 @@
+// Launches of the register-FFT time kernels (time_fft.cuh).
+#include <algorithm>
+
+#include "time_fft_dispatch.cuh"
+
+namespace aahrt {
+
+static FrameFn frame_pick(int L) {
+    switch (L) {
+        case 9: return frame_call<2>;
+        case 10: return frame_call<4>;
+        case 11: return frame_call<8>;
+        case 12: return frame_call<16>;
+        case 13: return frame_call<32>;
+        default: return nullptr;
+    }
+}
+
+template <int C>
+static size_t frame_most(int pairs, int nrows, int nfrac) {
+    return frame_smem<Frame<C>>(pairs, nrows, nfrac);
+}
+
+// Shared memory of the largest time kernel of frames of 2^L samples.
+static size_t frame_plan_smem(int L, int pairs, int nt, int ntau, int ns) {
+    const int nrows = std::max(nt, ntau), nfrac = std::max(nt, ns);
+    switch (L) {
+        case 9: return frame_most<2>(pairs, nrows, nfrac);
+        case 10: return frame_most<4>(pairs, nrows, nfrac);
+        case 11: return frame_most<8>(pairs, nrows, nfrac);
+        case 12: return frame_most<16>(pairs, nrows, nfrac);
+        default: return frame_most<32>(pairs, nrows, nfrac);
+    }
+}
+
+bool frame_serves(int L, int nt, int ntau, int ns, int max_smem) {
+    // (1 KB stays for the kernels' static shared memory)
+    return L >= 9 && L <= 13 && frame_plan_smem(L, 1, nt, ntau, ns) + 1024 <= (size_t)max_smem;
+}
+
+cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem) {
+    // 256 threads a block, fewer while blocks are fewer than SMs
+    const long long groups = std::min(p.ncg_model_blk, p.ncg_data_blk);
+    p.frame_pairs = std::max(1, 256 / (p.nfft / 16));
+    while (p.frame_pairs > 1 &&
+           (groups / p.frame_pairs < num_sms ||
+            frame_plan_smem(p.L, p.frame_pairs, p.nt, p.ntau, p.ns) + 1024 > (size_t)max_smem))
+        p.frame_pairs /= 2;
+    p.frame_ahead = (p.L <= 12 ? 3 : 1) * num_sms;       // by registers and shared memory
+    const FrameFn fn = frame_pick(p.L);
+    const FrameArgs none{};
+    cudaError_t e = cudaSuccess;
+    for (int op = 0; op < 3; ++op)
+        for (int model = 0; model < 2; ++model)
+            for (int epi = 0; epi < 3 && !e; ++epi)
+                e = fn(FrameCall{(FrameOp)op, model != 0, p.interp, epi, 1, nullptr, max_smem}, none,
+                       nullptr, nullptr, nullptr);
+    return e;
+}
+
+cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *in, void *out,
+                         const float *aux, const FistaArgs &fa, bool blocked, bool bound,
+                         cudaStream_t st) {
+    FrameArgs a;
+    a.groups = model_side ? (blocked ? p.cg_model_blk : p.cg_model_pair)
+                          : (blocked ? p.cg_data_blk : p.cg_data_pair);
+    a.ngroups = model_side ? p.ncg_model_blk : p.ncg_data_blk;
+    a.syn = model_side ? p.ST : p.U;
+    a.ana = model_side ? p.S : p.UT;
+    a.nrows = model_side ? p.ntau : p.nt;
+    // fractions: of S^T in a model synthesis, of U^T in a data analysis
+    a.nfrac = model_side ? (op == FRAME_R2C ? 0 : p.ns) : (op == FRAME_C2R ? 0 : p.nt);
+    a.frac = model_side ? p.frac_s : p.frac_u;
+    a.sc = FrameScatter{p.sc_i0, p.sc_n0};
+    a.ahead = p.frame_pairs == 1 ? p.frame_ahead : 0;
+    a.ns = p.ns;
+    a.nbins = p.nbins;
+    a.tw = p.tw_t;
+    a.fa = fa;
+    a.ybd = bound ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
+    return frame_pick(p.L)(FrameCall{(FrameOp)op, model_side, p.interp, epi, p.frame_pairs, st, 0}, a,
+                           in, out, aux);
+}
+
+}  // namespace aahrt

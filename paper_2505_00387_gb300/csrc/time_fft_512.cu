@@ -1,0 +1,8 @@
+// Register-FFT time kernels of 512-sample frames.
+#include "time_fft_dispatch.cuh"
+
+namespace aahrt {
+
+template cudaError_t frame_call<2>(const FrameCall &, const FrameArgs &, const void *, void *, const float *);
+
+}  // namespace aahrt

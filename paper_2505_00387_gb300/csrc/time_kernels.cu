@@ -1,4 +1,7 @@
-// Time-axis stages of the AAHRT (Algorithms 1 and 2, steps 1-2 and 4-5):
+// Time-axis stages of the AAHRT (Algorithms 1 and 2, steps 1-2 and 4-5) on
+// spectra whose columns or gathers are fastest: every plan's stages on natural
+// layouts (aahrt_apply_stage, the pull scan), and the operators of the plans
+// the bins-fastest kernels (time_fft.cuh) do not serve:
 //
 //   r2c: X[k][c] = sum_n (G in)[n][c] exp(-2 pi i k n / Nfft), k < nbins
 //        where G resamples each column: the time stretch S (model side,
@@ -42,10 +45,8 @@ constexpr int kPackBatch = 8;   // spectrum loads in flight per thread (c2r pack
 // Threads of a time-kernel block: 256 while two blocks fit in one SM's shared
 // memory, else 512 (one block per SM, e.g. the 8192-point frames of long
 // traces), so an SM keeps 16 warps in flight either way.  Both run under the
-// same 128-register cap.  Blocks of few samples (one radix-16 group per
-// thread would take under 128 threads) run 128.
-static int time_threads(size_t smem, int samples) {
-    if (samples <= 16 * 128) return 128;
+// same 128-register cap.
+static int time_threads(size_t smem) {
     return smem + 512 <= (size_t)kTimeSmemTwoBlocks ? kThreadsTime : kMaxThreadsTime;
 }
 
@@ -112,38 +113,12 @@ struct YBound {
     int nchunk, chunk_log;
 };
 
-// Where a column group's spectrum lies: element (bin k, column c) at
-// off + k ks + c cs, and how a block's threads walk it.  Bins-fastest spectra
-// (ks = 1) are walked bin by bin within a column pair, the others pair by pair
-// within a bin.
-struct SpecMap {
-    long long off, cs;
-    int ks, nbr;              // nbr: bins of one pair's walk (whole warps)
-    bool bins;
-    __device__ __forceinline__ SpecMap(const ColGroup &cg, int bins_fastest, int nbins, int nwalk)
-        : off(bins_fastest ? cg.bins_off : cg.spec_off), cs(bins_fastest ? nbins : 1),
-          ks(bins_fastest ? 1 : cg.ld_spec), nbr((nwalk + 31) & ~31), bins(bins_fastest) {}
-    template <int LP>
-    __device__ __forceinline__ void at(int idx, int *p, int *k) const {
-        if (bins) {
-            int q = 0;
-#pragma unroll
-            for (int u = 1; u < (1 << LP); ++u) q += idx >= u * nbr;
-            *p = q;
-            *k = idx - q * nbr;
-        } else {
-            *p = idx & ((1 << LP) - 1);
-            *k = idx >> LP;
-        }
-    }
-};
-
 template <int LP, int INTERP, bool TRANS>
 __device__ __forceinline__ void r2c_core(float2 *sm, const float *stg, const float *sfr,
                                          const ColGroup &cg, const DevResampler &rs,
                                          int nrow_in, const float2 *__restrict__ tw, int L,
                                          int nbins, float2 *__restrict__ out,
-                                         const YBound &ybd, int bins_fastest) {
+                                         const YBound &ybd) {
     constexpr int P = 1 << LP;
     const int N = 1 << L;
     const int ld = ld_interleaved(N);
@@ -188,8 +163,7 @@ __device__ __forceinline__ void r2c_core(float2 *sm, const float *stg, const flo
     block_fft<true, false, IBatch, true>(IBatch{sm, ld}, P, L, tw);
 
     // unpack the two real spectra: A = (Z_k + conj Z_{N-k})/2, B = (Z_k - conj Z_{N-k})/(2i)
-    const SpecMap map(cg, bins_fastest, nbins, nbins);
-    float2 *dst = out + map.off;
+    float2 *dst = out + cg.spec_off;
     const int npair = (cg.ncol + 1) >> 1;
     const bool bound = TRANS && ybd.max != nullptr;
     __shared__ unsigned s_ymax[128];
@@ -199,26 +173,25 @@ __device__ __forceinline__ void r2c_core(float2 *sm, const float *stg, const flo
     }
     // rows 16-byte aligned (even row stride and offset): a column pair's A and
     // B leave as one 16-byte store
-    const bool wide = !map.bins && ((cg.ld_spec | cg.spec_off) & 1) == 0;
-    const int total = map.bins ? P * map.nbr : P * nbins;
-    const int kend = ((total + blockDim.x - 1) / blockDim.x) * blockDim.x;
+    const bool wide = ((cg.ld_spec | cg.spec_off) & 1) == 0;
+    const int kend = ((P * nbins + blockDim.x - 1) / blockDim.x) * blockDim.x;
     for (int idx = threadIdx.x; idx < kend; idx += blockDim.x) {
-        int p, k;
-        map.at<LP>(idx, &p, &k);
+        const int p = idx & (P - 1);
+        const int k = idx >> LP;
         float amax = 0.f;
-        if (idx < total && k < nbins && p < npair) {
+        if (idx < P * nbins && p < npair) {
             const float2 zk = sm[p * ld + padi(brev_bits(k, L))];
             const float2 zn = sm[p * ld + padi(brev_bits((N - k) & (N - 1), L))];
             const float2 A = make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
             const float2 B = make_float2(0.5f * (zk.y + zn.y), -0.5f * (zk.x - zn.x));
-            const long long o = (long long)k * map.ks + 2 * p * map.cs;
+            const long long o = (long long)k * cg.ld_spec + 2 * p;
             amax = fabsf(A.x) + fabsf(A.y);
             if (2 * p + 1 < cg.ncol) {
                 if (wide)
                     *reinterpret_cast<float4 *>(dst + o) = make_float4(A.x, A.y, B.x, B.y);
                 else {
                     dst[o] = A;
-                    dst[o + map.cs] = B;
+                    dst[o + 1] = B;
                 }
                 amax = fmaxf(amax, fabsf(B.x) + fabsf(B.y));
             } else {
@@ -226,12 +199,11 @@ __device__ __forceinline__ void r2c_core(float2 *sm, const float *stg, const flo
             }
         }
         if (bound) {
-            // a warp's 32 / P (bins fastest: 32) bins lie inside one chunk
-            // (chunks of >= 64 bins)
+            // a warp's 32 / P bins lie inside one chunk (chunks of >= 64 bins)
 #pragma unroll
             for (int sh = 16; sh > 0; sh >>= 1)
                 amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, sh));
-            const int kw = map.bins ? (k & ~31) : (idx & ~31) >> LP;
+            const int kw = (idx & ~31) >> LP;
             if ((threadIdx.x & 31) == 0 && kw < nbins && amax > 0.f)
                 atomicMax(s_ymax + (kw >> ybd.chunk_log), __float_as_uint(amax));
         }
@@ -252,7 +224,7 @@ template <int LP, int INTERP, bool TRANS>
 __global__ void __launch_bounds__(kMaxThreadsTime, 1)
 r2c_kernel(const float *__restrict__ in, float2 *__restrict__ out,
            const ColGroup *__restrict__ groups, DevResampler rs, int nrow_in,
-           const float2 *__restrict__ tw, int L, int nbins, YBound ybd, int bins_fastest) {
+           const float2 *__restrict__ tw, int L, int nbins, YBound ybd) {
     constexpr int P = 1 << LP;
     extern __shared__ float4 smem_f4[];
     float2 *sm = reinterpret_cast<float2 *>(smem_f4);
@@ -282,8 +254,7 @@ r2c_kernel(const float *__restrict__ in, float2 *__restrict__ out,
         for (int idx = threadIdx.x; idx < rs.npos; idx += blockDim.x)
             sfr[idx] = __ldg(&rs.pos[idx].fr);
     __syncthreads();
-    r2c_core<LP, INTERP, TRANS>(sm, stg, sfr, cg, rs, nrow_in, tw, L, nbins, out, ybd,
-                                bins_fastest);
+    r2c_core<LP, INTERP, TRANS>(sm, stg, sfr, cg, rs, nrow_in, tw, L, nbins, out, ybd);
 }
 
 // The c2r pipeline of one column group.  With STAGE, the epilogue's real
@@ -296,13 +267,12 @@ __device__ __forceinline__ void c2r_core(float2 *sm, float *sfr, const float2 *_
                                          const float *__restrict__ aux, const FistaArgs &fa,
                                          const ColGroup &cg, const DevResampler &rs, int n_in,
                                          const float2 *__restrict__ tw, int L, int nbins,
-                                         float *stg, int bins_fastest) {
+                                         float *stg) {
     constexpr int P = 1 << LP;
     const int N = 1 << L;
     const int half = N >> 1;
     const int ld = ld_interleaved(N);
-    const SpecMap map(cg, bins_fastest, nbins, half + 1);
-    const float2 *src = in + map.off;
+    const float2 *src = in + cg.spec_off;
     const int npair = (cg.ncol + 1) >> 1;
 
     if (TRANS)
@@ -311,19 +281,19 @@ __device__ __forceinline__ void c2r_core(float2 *sm, float *sfr, const float2 *_
     // pack Z = A + iB over the full frame, bit-reversed for the DIT pass;
     // kPackBatch rounds of loads are issued before any is used, so each
     // thread keeps that many spectrum reads in flight
-    const int total = map.bins ? P * map.nbr : P * (half + 1);
+    const int total = P * (half + 1);
     // rows 16-byte aligned: a column pair's A and B arrive as one 16-byte load
-    const bool wide = !map.bins && ((cg.ld_spec | cg.spec_off) & 1) == 0;
+    const bool wide = ((cg.ld_spec | cg.spec_off) & 1) == 0;
     for (int base = threadIdx.x; base < total; base += kPackBatch * blockDim.x) {
         float2 A[kPackBatch], B[kPackBatch];
 #pragma unroll
         for (int u = 0; u < kPackBatch; ++u) {
             const int idx = base + u * blockDim.x;
-            int p, k;
-            map.at<LP>(idx, &p, &k);
+            const int p = idx & (P - 1);
+            const int k = idx >> LP;
             A[u] = B[u] = make_float2(0.f, 0.f);
             if (idx < total && k < nbins && p < npair) {
-                const long long o = (long long)k * map.ks + 2 * p * map.cs;
+                const long long o = (long long)k * cg.ld_spec + 2 * p;
                 // the fused kernel rewrites the spectrum later: plain loads there
                 if (wide && 2 * p + 1 < cg.ncol) {
                     const float4 *q4 = reinterpret_cast<const float4 *>(src + o);
@@ -332,8 +302,7 @@ __device__ __forceinline__ void c2r_core(float2 *sm, float *sfr, const float2 *_
                     B[u] = make_float2(v.z, v.w);
                 } else {
                     A[u] = STAGE ? src[o] : __ldg(src + o);
-                    if (2 * p + 1 < cg.ncol)
-                        B[u] = STAGE ? src[o + map.cs] : __ldg(src + o + map.cs);
+                    if (2 * p + 1 < cg.ncol) B[u] = STAGE ? src[o + 1] : __ldg(src + o + 1);
                 }
             }
         }
@@ -341,9 +310,8 @@ __device__ __forceinline__ void c2r_core(float2 *sm, float *sfr, const float2 *_
         for (int u = 0; u < kPackBatch; ++u) {
             const int idx = base + u * blockDim.x;
             if (idx >= total) break;
-            int p, k;
-            map.at<LP>(idx, &p, &k);
-            if (k > half) continue;
+            const int p = idx & (P - 1);
+            const int k = idx >> LP;
             float2 a = A[u], b = B[u];
             if (k == 0) { a.y = 0.f; b.y = 0.f; }
             const float2 zk = make_float2(a.x - b.y, a.y + b.x);   // A + iB
@@ -465,14 +433,14 @@ __global__ void __launch_bounds__(kMaxThreadsTime, 1)
 c2r_kernel(const float2 *__restrict__ in, float *__restrict__ out,
            const float *__restrict__ aux, FistaArgs fa,
            const ColGroup *__restrict__ groups, DevResampler rs, int n_in,
-           const float2 *__restrict__ tw, int L, int nbins, int bins_fastest) {
+           const float2 *__restrict__ tw, int L, int nbins) {
     constexpr int P = 1 << LP;
     extern __shared__ float4 smem_f4[];
     float2 *sm = reinterpret_cast<float2 *>(smem_f4);
     const ColGroup cg = groups[blockIdx.x];
     float *sfr = reinterpret_cast<float *>(sm + P * ld_interleaved(1 << L));
     c2r_core<LP, INTERP, TRANS, EPI, false>(sm, sfr, in, out, aux, fa, cg, rs, n_in, tw, L,
-                                            nbins, nullptr, bins_fastest);
+                                            nbins, nullptr);
 }
 
 // One FISTA half-iteration's two time stages on the same column group, fused:
@@ -488,7 +456,7 @@ __global__ void __launch_bounds__(kMaxThreadsTime, 1)
 c2r_r2c_kernel(float2 *spec, const float *__restrict__ aux, FistaArgs fa,
                const ColGroup *__restrict__ groups, DevResampler rs_syn, int n_in,
                DevResampler rs_ana, int nrow_mid, const float2 *__restrict__ tw, int L,
-               int nbins, YBound ybd, int bins_fastest) {
+               int nbins, YBound ybd) {
     constexpr int P = 1 << LP;
     constexpr bool ANA_TRANS = !SYN_TRANS;
     extern __shared__ float4 smem_f4[];
@@ -503,28 +471,27 @@ c2r_r2c_kernel(float2 *spec, const float *__restrict__ aux, FistaArgs fa,
                      cg.ld_real);
     cp_async_commit();
     c2r_core<LP, INTERP, SYN_TRANS, EPI, true>(sm, sfr, spec, nullptr, aux, fa, cg, rs_syn, n_in,
-                                               tw, L, nbins, stg, bins_fastest);
+                                               tw, L, nbins, stg);
     __syncthreads();
     if (ANA_TRANS) {
         for (int idx = threadIdx.x; idx < rs_ana.npos; idx += blockDim.x)
             sfr[idx] = __ldg(&rs_ana.pos[idx].fr);
         __syncthreads();
     }
-    r2c_core<LP, INTERP, ANA_TRANS>(sm, stg, sfr, cg, rs_ana, nrow_mid, tw, L, nbins, spec, ybd,
-                                    bins_fastest);
+    r2c_core<LP, INTERP, ANA_TRANS>(sm, stg, sfr, cg, rs_ana, nrow_mid, tw, L, nbins, spec, ybd);
 }
 
 // ------------------------------------------------------------- dispatch
 template <int LP, int INTERP>
 static void r2c_launch(bool model_side, int grid, size_t smem, cudaStream_t st, const float *in,
                        float2 *out, const ColGroup *cg, DevResampler rs, int nrow_in,
-                       const float2 *tw, int L, int nbins, bool bins, YBound ybd = YBound{}) {
+                       const float2 *tw, int L, int nbins, YBound ybd = YBound{}) {
     if (model_side)
-        r2c_kernel<LP, INTERP, false><<<grid, time_threads(smem, 1 << (L + LP)), smem, st>>>(
-            in, out, cg, rs, nrow_in, tw, L, nbins, YBound{}, bins);
+        r2c_kernel<LP, INTERP, false><<<grid, time_threads(smem), smem, st>>>(in, out, cg, rs, nrow_in,
+                                                                        tw, L, nbins, YBound{});
     else
-        r2c_kernel<LP, INTERP, true><<<grid, time_threads(smem, 1 << (L + LP)), smem, st>>>(
-            in, out, cg, rs, nrow_in, tw, L, nbins, ybd, bins);
+        r2c_kernel<LP, INTERP, true><<<grid, time_threads(smem), smem, st>>>(in, out, cg, rs, nrow_in,
+                                                                       tw, L, nbins, ybd);
 }
 
 // The bound table of the data spectrum, cleared for the analysis about to
@@ -539,13 +506,13 @@ template <int LP, int INTERP, int EPI>
 static void c2r_launch(bool model_side, int grid, size_t smem, cudaStream_t st,
                        const float2 *in, float *out, const float *aux, FistaArgs fa,
                        const ColGroup *cg, DevResampler rs, int n_in, const float2 *tw, int L,
-                       int nbins, bool bins) {
+                       int nbins) {
     if (model_side)
-        c2r_kernel<LP, INTERP, true, EPI><<<grid, time_threads(smem, 1 << (L + LP)), smem, st>>>(
-            in, out, aux, fa, cg, rs, n_in, tw, L, nbins, bins);
+        c2r_kernel<LP, INTERP, true, EPI><<<grid, time_threads(smem), smem, st>>>(
+            in, out, aux, fa, cg, rs, n_in, tw, L, nbins);
     else
-        c2r_kernel<LP, INTERP, false, EPI><<<grid, time_threads(smem, 1 << (L + LP)), smem, st>>>(
-            in, out, aux, fa, cg, rs, n_in, tw, L, nbins, bins);
+        c2r_kernel<LP, INTERP, false, EPI><<<grid, time_threads(smem), smem, st>>>(
+            in, out, aux, fa, cg, rs, n_in, tw, L, nbins);
 }
 
 #define AAHRT_LP_SWITCH(LPV, STMT)                      \
@@ -561,7 +528,6 @@ static void c2r_launch(bool model_side, int grid, size_t smem, cudaStream_t st,
 
 cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
                        cudaStream_t st, bool blocked, bool natural) {
-    const bool bins = p.bins_fastest && !natural;
     const ColGroup *cg = model_side ? (blocked ? p.cg_model_blk : p.cg_model)
                                     : (blocked ? p.cg_data_blk : p.cg_data);
     const int n = model_side ? p.ncg_model : p.ncg_data;
@@ -575,8 +541,15 @@ cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
         if (e) return e;
     }
     prof_begin(p, stage, st);
+    if (p.bins_fastest && !natural) {
+        const cudaError_t e = launch_frame(p, 0, model_side, EPI_STORE, in, out, nullptr,
+                                           FistaArgs{}, blocked, !model_side, st);
+        prof_end(p, st);
+        p.launches[stage]++;
+        return e;
+    }
     AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (r2c_launch<LPc, IPc>(
-        model_side, n, smem, st, in, out, cg, rs, nrow_in, p.tw_t, p.L, p.nbins, bins, yb))));
+        model_side, n, smem, st, in, out, cg, rs, nrow_in, p.tw_t, p.L, p.nbins, yb))));
     prof_end(p, st);
     p.launches[stage]++;
     return cudaGetLastError();
@@ -585,7 +558,6 @@ cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
 cudaError_t launch_c2r(Plan &p, bool model_side, const float2 *in, float *out,
                        int epi, const float *aux, FistaArgs fa, cudaStream_t st, bool blocked,
                        bool natural) {
-    const bool bins = p.bins_fastest && !natural;
     const ColGroup *cg = model_side ? (blocked ? p.cg_model_blk : p.cg_model)
                                     : (blocked ? p.cg_data_blk : p.cg_data);
     const int n = model_side ? p.ncg_model : p.ncg_data;
@@ -594,21 +566,25 @@ cudaError_t launch_c2r(Plan &p, bool model_side, const float2 *in, float *out,
     const size_t smem = model_side ? p.smem_c2r_model : p.smem_c2r_data;
     const int stage = model_side ? 5 : 2;
     prof_begin(p, stage, st);
+    if (p.bins_fastest && !natural) {
+        const cudaError_t e = launch_frame(p, 1, model_side, epi, in, out, aux, fa, blocked, false,
+                                           st);
+        prof_end(p, st);
+        p.launches[stage]++;
+        return e;
+    }
     switch (epi) {
         case EPI_RESIDUAL:
             AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (c2r_launch<LPc, IPc, EPI_RESIDUAL>(
-                model_side, n, smem, st, in, out, aux, fa, cg, rs, n_in, p.tw_t, p.L, p.nbins,
-                bins))));
+                model_side, n, smem, st, in, out, aux, fa, cg, rs, n_in, p.tw_t, p.L, p.nbins))));
             break;
         case EPI_FISTA:
             AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (c2r_launch<LPc, IPc, EPI_FISTA>(
-                model_side, n, smem, st, in, out, aux, fa, cg, rs, n_in, p.tw_t, p.L, p.nbins,
-                bins))));
+                model_side, n, smem, st, in, out, aux, fa, cg, rs, n_in, p.tw_t, p.L, p.nbins))));
             break;
         default:
             AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (c2r_launch<LPc, IPc, EPI_STORE>(
-                model_side, n, smem, st, in, out, aux, fa, cg, rs, n_in, p.tw_t, p.L, p.nbins,
-                bins))));
+                model_side, n, smem, st, in, out, aux, fa, cg, rs, n_in, p.tw_t, p.L, p.nbins))));
             break;
     }
     prof_end(p, st);
@@ -645,19 +621,25 @@ cudaError_t launch_c2r_r2c(Plan &p, bool model_side, float2 *spec, const float *
         if (e) return e;
     }
     prof_begin(p, stage, st);
+    if (p.bins_fastest) {
+        const cudaError_t e = launch_frame(p, 2, model_side, 0, spec, spec, aux, fa, true,
+                                           !model_side, st);
+        prof_end(p, st);
+        p.launches[stage]++;
+        return e;
+    }
     if (model_side) {
         AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (
-            c2r_r2c_kernel<LPc, IPc, true, EPI_FISTA><<<n, time_threads(p.smem_fused_model, 1 << (p.L + LPc)),
+            c2r_r2c_kernel<LPc, IPc, true, EPI_FISTA><<<n, time_threads(p.smem_fused_model),
                                                          p.smem_fused_model, st>>>(
                 spec, nullptr, fa, cg, p.ST, p.ns, p.S, p.ntau, p.tw_t, p.L, p.nbins,
-                YBound{}, p.bins_fastest))));
+                YBound{}))));
     } else {
         AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (
-            c2r_r2c_kernel<LPc, IPc, false, EPI_RESIDUAL><<<n, time_threads(p.smem_r2c_data, 1 << (p.L + LPc)),
+            c2r_r2c_kernel<LPc, IPc, false, EPI_RESIDUAL><<<n, time_threads(p.smem_r2c_data),
                                                            p.smem_r2c_data,
                                                            st>>>(
-                spec, aux, FistaArgs{}, cg, p.U, p.ns, p.UT, p.nt, p.tw_t, p.L, p.nbins, yb,
-                p.bins_fastest))));
+                spec, aux, FistaArgs{}, cg, p.U, p.ns, p.UT, p.nt, p.tw_t, p.L, p.nbins, yb))));
     }
     prof_end(p, st);
     p.launches[stage]++;
@@ -680,7 +662,7 @@ cudaError_t launch_stretch_data(Plan &p, const float *d, float2 *Y, cudaStream_t
     prof_begin(p, 3, st);
     AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (r2c_launch<LPc, IPc>(
         true, p.ncg_data, p.smem_r2c_model, st, d, Y, p.cg_data, p.S, p.nt, p.tw_t, p.L,
-        p.nbins, false))));
+        p.nbins))));
     prof_end(p, st);
     p.launches[3]++;
     return cudaGetLastError();
@@ -692,7 +674,7 @@ cudaError_t launch_unstretch_model(Plan &p, const float2 *X, float *m, cudaStrea
     prof_begin(p, 5, st);
     AAHRT_LP_SWITCH(p.lp, AAHRT_INTERP_SWITCH(p.interp, (c2r_launch<LPc, IPc, EPI_STORE>(
         false, p.ncg_model, p.smem_c2r_data, st, X, m, nullptr, FistaArgs{}, p.cg_model, p.U,
-        p.ns, p.tw_t, p.L, p.nbins, false))));
+        p.ns, p.tw_t, p.L, p.nbins))));
     prof_end(p, st);
     p.launches[5]++;
     return cudaGetLastError();

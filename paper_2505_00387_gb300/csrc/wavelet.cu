@@ -53,7 +53,7 @@ cudaError_t launch_wavelet(Plan &p, int mode, const float *in, float *out, const
                            cudaStream_t st, bool blocked) {
     const ColGroup *groups = blocked ? p.cg_data_blk : p.cg_data;
     const size_t smem = (size_t)(((p.nw + 3) & ~3) + p.nt * 2 * p.pairs) * sizeof(float);
-    const int grid = p.ncg_data;
+    const int grid = blocked ? p.ncg_data_blk : p.ncg_data;
     switch (mode) {
         case WAV_CONV:
             wavelet_kernel<WAV_CONV><<<grid, 256, smem, st>>>(in, out, aux, groups, p.nt, p.wav,
