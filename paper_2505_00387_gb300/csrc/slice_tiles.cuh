@@ -260,28 +260,25 @@ tile_fwd_kernel(const TileArgs a, const float2 *__restrict__ X, float2 *__restri
 }
 
 // ------------------------------------------------------------- adjoint
-// A grid row holds TB real parts, then TB imaginary parts (32-bit fixed point
-// while spreading, floats between the two DFT steps).  With TB = 16 a warp
-// spreads two traces: its halves take the real and the imaginary plane in
+// A grid row holds TB real parts, then TB imaginary parts in 32-bit fixed point
+// while spreading, and TB complex floats between the two DFT steps (every row
+// is read, rewritten and cleared by the lanes of one warp).  With TB = 16 a
+// warp spreads two traces: its halves take the real and the imaginary plane in
 // opposite order, so their rows never share a bank.
 template <int TB>
 struct PlanePair {
-    float *first, *second;       // the plane this half warp takes first, and the other
+    const int *first, *second;   // the plane this half warp takes first, and the other
     bool swap;
-    __device__ __forceinline__ explicit PlanePair(float *p)
+    __device__ __forceinline__ explicit PlanePair(const int *p)
         : first(p), second(p + TB), swap(TB == 16 && (threadIdx.x & 16)) {
         if (swap) {
             first = p + TB;
             second = p;
         }
     }
-    __device__ __forceinline__ float2 load(int off) const {
-        const float x = first[off], y = second[off];
-        return swap ? make_float2(y, x) : make_float2(x, y);
-    }
-    __device__ __forceinline__ void store(int off, float2 v) const {
-        first[off] = swap ? v.y : v.x;
-        second[off] = swap ? v.x : v.y;
+    __device__ __forceinline__ int2 load(int off) const {
+        const int x = first[off], y = second[off];
+        return swap ? make_int2(y, x) : make_int2(x, y);
     }
 };
 
@@ -303,19 +300,18 @@ __device__ __forceinline__ void tile_spread(int *G, const float *phi, int row, f
 // and cleared) -> inverse radix-R, conjugate twiddles, floats in rows
 // p1 + 16 n2.  R = 32 by two threads, one for each parity of n2.
 template <class T>
-__device__ __forceinline__ void tile_adj_step1(float *G, int sub, int bin, const float2 *s_tw,
+__device__ __forceinline__ void tile_adj_step1(float2 *G, int sub, int bin, const float2 *s_tw,
                                                float ifx) {
-    constexpr int TB = T::TB, R = T::R, WRAP = T::NOS * 2 * TB;
-    auto fixed = [&](const PlanePair<TB> &pl, int p1, int n, bool clear) {
-        float2 raw = pl.load(n * 32 * TB);
-        int re = __float_as_int(raw.x), im = __float_as_int(raw.y);
+    constexpr int TB = T::TB, R = T::R;
+    // row n of the column in fixed point
+    auto fixed = [&](const PlanePair<TB> &pl, int p1, int n) {
+        int2 v = pl.load(n * 32 * TB);
         if (n == 0 && p1 < T::W - 1) {
-            raw = pl.load(WRAP);
-            re += __float_as_int(raw.x);
-            im += __float_as_int(raw.y);
-            if (clear) pl.store(WRAP, make_float2(0.f, 0.f));
+            const int2 u = pl.load(T::NOS * 2 * TB);
+            v.x += u.x;
+            v.y += u.y;
         }
-        return make_float2((float)re * ifx, (float)im * ifx);
+        return make_float2((float)v.x * ifx, (float)v.y * ifx);
     };
     auto twiddled = [&](float2 v, int n2, int p1) {
         const float2 w = s_tw[(n2 << 4) + p1];
@@ -323,31 +319,35 @@ __device__ __forceinline__ void tile_adj_step1(float *G, int sub, int bin, const
     };
     if constexpr (T::LR == 5) {
         const int p1 = sub & 15, b = sub >> 4;           // NSUB = 32
-        const PlanePair<TB> pl(G + p1 * 2 * TB + bin);
+        const PlanePair<TB> pl(reinterpret_cast<const int *>(G + p1 * TB) + bin);
         float2 v[16];
-        half_of_32<true>(v, b, s_tw, [&](int n) { return fixed(pl, p1, n, false); });
+        half_of_32<true>(v, b, s_tw, [&](int n) { return fixed(pl, p1, n); });
         dif_network<4, true>(v);
         __syncthreads();
-        if (b == 0 && p1 < T::W - 1) pl.store(WRAP, make_float2(0.f, 0.f));
+        float2 *col = G + p1 * TB + bin;
+        if (b == 0 && p1 < T::W - 1) col[T::NOS * TB] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int m = 0; m < 16; ++m) {
             const int n2 = 2 * rev_bits_c<4>(m) + b;
-            pl.store(n2 * 32 * TB, twiddled(v[m], n2, p1));
+            col[n2 * 16 * TB] = twiddled(v[m], n2, p1);
         }
     } else {
 #pragma unroll
         for (int p0 = 0; p0 < 16; p0 += T::NSUB) {
             const int p1 = p0 + sub;
             if (T::NSUB > 16 && p1 >= 16) break;
-            const PlanePair<TB> pl(G + p1 * 2 * TB + bin);
+            const PlanePair<TB> pl(reinterpret_cast<const int *>(G + p1 * TB) + bin);
             float2 v[R];
 #pragma unroll
-            for (int n = 0; n < R; ++n) v[n] = fixed(pl, p1, n, true);
+            for (int n = 0; n < R; ++n) v[n] = fixed(pl, p1, n);
             dif_network<T::LR, true>(v);
+            float2 *col = G + p1 * TB + bin;
+            __syncwarp();        // the row's lanes have read it
+            if (p1 < T::W - 1) col[T::NOS * TB] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int m = 0; m < R; ++m) {
                 const int n2 = rev_bits_c<T::LR>(m);
-                pl.store(n2 * 32 * TB, n2 == 0 ? v[m] : twiddled(v[m], n2, p1));
+                col[n2 * 16 * TB] = n2 == 0 ? v[m] : twiddled(v[m], n2, p1);
             }
         }
     }
@@ -356,19 +356,19 @@ __device__ __forceinline__ void tile_adj_step1(float *G, int sub, int bin, const
 // Adjoint, second step: rows p1 + 16 n2 (cleared once read) -> inverse radix-16,
 // deapodised curvatures of slice j.
 template <class T>
-__device__ __forceinline__ void tile_adj_step2(const TileArgs &a, float *G, int sub, int bin,
+__device__ __forceinline__ void tile_adj_step2(const TileArgs &a, float2 *G, int sub, int bin,
                                                const float *s_dec, float2 *__restrict__ Xc, int j,
                                                bool live) {
     constexpr int TB = T::TB, R = T::R;
     const long long sl = (long long)a.ntheta * a.nbins;
     const bool centred = a.nq <= T::NOS / 2;
     for (int n2 = sub; n2 < R; n2 += T::NSUB) {
-        const PlanePair<TB> pl(G + (n2 << 4) * 2 * TB + bin);
+        float2 *col = G + (n2 << 4) * TB + bin;
         float2 v[16];
 #pragma unroll
         for (int p1 = 0; p1 < 16; ++p1) {
-            v[p1] = pl.load(p1 * 2 * TB);
-            pl.store(p1 * 2 * TB, make_float2(0.f, 0.f));
+            v[p1] = col[p1 * TB];
+            col[p1 * TB] = make_float2(0.f, 0.f);
         }
         dif_network<4, true>(v);
         float2 *p = Xc + (long long)j * a.nbins + (n2 + a.cq) * sl;
@@ -390,14 +390,14 @@ template <class T>
 __global__ void __launch_bounds__(T::THREADS, T::MINB)
 tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restrict__ X) {
     extern __shared__ float4 smem_f4[];
-    constexpr int W = T::W, TB = T::TB, NSUB = T::NSUB, GRID = T::ROWS * 2 * TB;
+    constexpr int W = T::W, TB = T::TB, NSUB = T::NSUB, GRID = T::ROWS * TB;
     __shared__ long long s_item;
-    float *buf = reinterpret_cast<float *>(smem_f4);
-    float2 *s_tw = reinterpret_cast<float2 *>(buf + 2 * GRID);
+    float2 *buf = reinterpret_cast<float2 *>(smem_f4);
+    float2 *s_tw = buf + 2 * GRID;
     float *s_dec = reinterpret_cast<float *>(s_tw + T::NOS);
     tile_tables<T>(a, s_tw, s_dec);
     // the grids start cleared, and the last reader of a row clears it
-    for (int i = threadIdx.x; i < 2 * GRID; i += T::THREADS) buf[i] = 0.f;
+    for (int i = threadIdx.x; i < 2 * GRID; i += T::THREADS) buf[i] = make_float2(0.f, 0.f);
     const int bin = threadIdx.x & (TB - 1);
     const int sub = threadIdx.x / TB;
     for (;;) {
@@ -436,17 +436,20 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
             int *G0 = reinterpret_cast<int *>(buf + cur * GRID);
             int *G1 = reinterpret_cast<int *>(buf + (cur ^ 1) * GRID);
             if (live && t0 + sub < t1) {
-                // a trace's record and y are loaded ahead of its use
-                TraceGeo nxt = geo[t0 + sub];
+                // a trace's record is loaded two traces ahead of its use, its y
+                // (found by the record) one ahead
+                TraceGeo nxt = geo[t0 + sub], far{};
+                if (t0 + sub + NSUB < t1) far = geo[t0 + sub + NSUB];
                 float2 ynxt = __ldg(Yc + (long long)nxt.col * a.nbins);
                 for (int t = t0 + sub; t < t1; t += NSUB) {
                     const TraceGeo tr = nxt;
                     const float2 y = ynxt;
-                    if (t + NSUB < t1) nxt = geo[t + NSUB];
+                    nxt = far;
+                    if (t + NSUB < t1) ynxt = __ldg(Yc + (long long)nxt.col * a.nbins);
+                    if (t + 2 * NSUB < t1) far = geo[t + 2 * NSUB];
                     const TapSet ts = trace_taps<W>(tr.A, tr.B, (unsigned)kb, T::LR + 4);
                     float phi[W];
                     es_weights<W>(a.poly, ts.g, phi);
-                    if (t + NSUB < t1) ynxt = __ldg(Yc + (long long)nxt.col * a.nbins);
                     float sn, cs;
                     phase_cs(ts.ph, &sn, &cs);
                     // scale * y * exp(+2 pi i ph)
@@ -465,7 +468,7 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
                     for (int l = sub; l < a.nq; l += NSUB)
                         Xc[((long long)l * a.ntheta + j) * a.nbins] = make_float2(0.f, 0.f);
             } else if (own0) {
-                float *G = buf + cur * GRID;
+                float2 *G = buf + cur * GRID;
                 const float ifx = bound0 > 0.f ? bound0 * 9.3132257461547852e-10f : 0.f;   // 1/fx0
                 tile_adj_step1<T>(G, sub, bin, s_tw, ifx);
                 __syncthreads();
