@@ -297,6 +297,9 @@ cudaError_t configure_tc_kernels(Plan &p, int num_sms, int max_smem);
 // 1 out = aux - W in, 2 out = W^T in
 cudaError_t launch_wavelet(Plan &p, int mode, const float *in, float *out, const float *aux,
                            cudaStream_t st, bool blocked);
+// A work counter of the bins-fastest slice kernels is followed, kDoneSlot
+// further on, by the count of finished blocks; the last block clears both.
+constexpr int kDoneSlot = 2;
 // device error flag of the tensor-core kernels (a timed-out wait), in Plan::counters
 constexpr int kTcErrSlot = 8;
 

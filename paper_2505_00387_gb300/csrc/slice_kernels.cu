@@ -425,19 +425,21 @@ cudaError_t launch_slice(Plan &p, bool adjoint, const float2 *in, float2 *out,
     const int slot = adjoint ? 1 : 0;
     const int stage = adjoint ? 4 : 1;
     int *ctr = counter ? counter : p.counters + slot;
-    cudaError_t e = cudaMemsetAsync(ctr, 0, sizeof(int), st);
-    if (e) return e;
-    if (p.precision == 1 || p.slice_interp == AAHRT_SLICE_DIRECT) {
+    cudaError_t e = cudaSuccess;
+    if (p.bins_fastest) {
+        // the plan's own counter is left cleared by every launch
+        if (counter && (e = cudaMemsetAsync(ctr, 0, (kDoneSlot + 1) * sizeof(int), st))) return e;
         prof_begin(p, stage, st);
-        e = p.precision == 1 ? launch_slice_tc(p, adjoint, in, out, st, ctr)
-                             : launch_slice_direct(p, adjoint, in, out, st, ctr);
+        e = launch_slice_tiles(p, adjoint, in, out, st, ctr);
         prof_end(p, st);
         p.launches[stage]++;
         return e;
     }
-    if (p.bins_fastest) {
+    if ((e = cudaMemsetAsync(ctr, 0, sizeof(int), st))) return e;
+    if (p.precision == 1 || p.slice_interp == AAHRT_SLICE_DIRECT) {
         prof_begin(p, stage, st);
-        e = launch_slice_tiles(p, adjoint, in, out, st, ctr);
+        e = p.precision == 1 ? launch_slice_tc(p, adjoint, in, out, st, ctr)
+                             : launch_slice_direct(p, adjoint, in, out, st, ctr);
         prof_end(p, st);
         p.launches[stage]++;
         return e;

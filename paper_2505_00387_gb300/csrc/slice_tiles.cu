@@ -26,6 +26,7 @@ static TileArgs tile_args(const Plan &p, int *counter) {
     a.phicap = (float)p.phicap;
     a.ymax = p.ymax;
     a.wsum = p.wsum;
+    a.ncube = p.ncube;
     a.nychunk = p.nychunk;
     a.ychunk_log = p.ychunk_log;
     a.poly = p.poly;

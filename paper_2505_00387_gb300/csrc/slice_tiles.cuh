@@ -39,9 +39,9 @@ struct TileArgs {
     int nbins, ntiles, nq, ntheta, nos, Lq, cq;
     float scale;
     float phicap;                          // bound on one kernel weight
-    const unsigned *__restrict__ ymax;
+    unsigned *ymax;
     const float *__restrict__ wsum;
-    int nychunk, ychunk_log;
+    int ncube, nychunk, ychunk_log;
     EsPoly poly;
 };
 
@@ -72,6 +72,20 @@ __device__ __forceinline__ void tile_tables(const TileArgs &a, float2 *s_tw, flo
         const int l = (i + a.cq) & (T::NOS - 1);
         s_dec[i] = l < a.nq ? __ldg(a.dec + l) : 0.f;
     }
+}
+
+// The block's work is done (thread 0 has drawn its last item): the last block
+// of the grid returns true in every thread and clears the work counter, so the
+// next launch finds it cleared without a memset between the kernels.
+__device__ __forceinline__ bool tile_last_block(int *counter) {
+    __shared__ int s_last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(counter + kDoneSlot, 1) == (int)gridDim.x - 1;
+        if (s_last) counter[0] = counter[kDoneSlot] = 0;
+    }
+    __syncthreads();
+    return s_last != 0;
 }
 
 // acc + w * g
@@ -165,7 +179,9 @@ __device__ __forceinline__ void tile_fwd_grid(const TileArgs &a, const float2 *_
         for (int m = 0; m < 16; ++m) {
             v[m] = make_float2(0.f, 0.f);
             if (m >= 4 && m < 12 && centred) continue;
-            if (m < 8 ? m * R < hi : m * R >= lo) v[m] = __ldg(p + (m < 8 ? m * R : m * R - T::NOS) * sl);
+            // (past L1, which keeps the trace records)
+            if (m < 8 ? m * R < hi : m * R >= lo)
+                v[m] = __ldcg(p + (m < 8 ? m * R : m * R - T::NOS) * sl);
         }
 #pragma unroll
         for (int m = 0; m < 16; ++m) {
@@ -257,6 +273,7 @@ tile_fwd_kernel(const TileArgs a, const float2 *__restrict__ X, float2 *__restri
         }
         __syncthreads();             // s_item is rewritten next
     }
+    tile_last_block(a.counter);
 }
 
 // ------------------------------------------------------------- adjoint
@@ -415,8 +432,8 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
         const int *ss = a.slice_start + g.ss_off;
         // fixed-point scale of a slice: 2^30 over the largest value a grid
         // point can reach (every trace of the slice at most phicap there)
-        const float M = live ? __uint_as_float(__ldg(a.ymax + (long long)g.cube * a.nychunk +
-                                                     (kb >> a.ychunk_log)))
+        const float M = live ? __uint_as_float(__ldcg(a.ymax + (long long)g.cube * a.nychunk +
+                                                      (kb >> a.ychunk_log)))
                              : 0.f;
         const float *ws = a.wsum + (long long)g.cube * a.ntheta;
         int cur = 0;
@@ -440,12 +457,12 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
                 // (found by the record) one ahead
                 TraceGeo nxt = geo[t0 + sub], far{};
                 if (t0 + sub + NSUB < t1) far = geo[t0 + sub + NSUB];
-                float2 ynxt = __ldg(Yc + (long long)nxt.col * a.nbins);
+                float2 ynxt = __ldcg(Yc + (long long)nxt.col * a.nbins);
                 for (int t = t0 + sub; t < t1; t += NSUB) {
                     const TraceGeo tr = nxt;
                     const float2 y = ynxt;
                     nxt = far;
-                    if (t + NSUB < t1) ynxt = __ldg(Yc + (long long)nxt.col * a.nbins);
+                    if (t + NSUB < t1) ynxt = __ldcg(Yc + (long long)nxt.col * a.nbins);
                     if (t + 2 * NSUB < t1) far = geo[t + 2 * NSUB];
                     const TapSet ts = trace_taps<W>(tr.A, tr.B, (unsigned)kb, T::LR + 4);
                     float phi[W];
@@ -479,6 +496,9 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
         }
         __syncthreads();             // s_item is rewritten next
     }
+    // the bound table is read: clear it for the analysis that writes the next Y
+    if (tile_last_block(a.counter))
+        for (int i = threadIdx.x; i < a.ncube * a.nychunk; i += T::THREADS) a.ymax[i] = 0u;
 }
 
 }  // namespace aahrt
