@@ -172,6 +172,7 @@ struct Plan {
     int ncg_model_blk = 0, ncg_data_blk = 0, blk_lp = 0;
     int frame_pairs = 0;           // column pairs per register-FFT block
     int frame_ahead = 0;           // such blocks resident on the device
+    int frame_seq_model = 1, frame_seq_data = 1;   // pairs an analysis block takes in turn
     float *frac_s = nullptr, *frac_u = nullptr;   // the resamplers' fractions alone
     int sc_i0 = 0, sc_n0 = 0;      // U^T: rows scattered from sc_i0, gathered below sc_n0
     long long mblk_len = 0, dblk_len = 0;

@@ -18,7 +18,18 @@ static FrameFn frame_pick(int L) {
 
 template <int C>
 static size_t frame_most(int pairs, int nrows, int nfrac) {
-    return frame_smem<Frame<C>>(pairs, nrows, nfrac);
+    return frame_smem<Frame<C>>(pairs, 1, nrows, nfrac);
+}
+
+// Shared memory of an analysis block of one pair taking seq pairs in turn.
+static size_t frame_analysis_smem(int L, int seq, int nrows, int nfrac) {
+    switch (L) {
+        case 9: return frame_smem<Frame<2>>(1, seq, nrows, nfrac);
+        case 10: return frame_smem<Frame<4>>(1, seq, nrows, nfrac);
+        case 11: return frame_smem<Frame<8>>(1, seq, nrows, nfrac);
+        case 12: return frame_smem<Frame<16>>(1, seq, nrows, nfrac);
+        default: return frame_smem<Frame<32>>(1, seq, nrows, nfrac);
+    }
 }
 
 // Shared memory of the largest time kernel of frames of 2^L samples.
@@ -46,6 +57,22 @@ cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem) {
            (groups / p.frame_pairs < num_sms ||
             frame_plan_smem(p.L, p.frame_pairs, p.nt, p.ntau, p.ns) + 1024 > (size_t)max_smem))
         p.frame_pairs /= 2;
+    // pairs an analysis block of one pair takes in turn: as many as cost at most
+    // 3 % more rounds of resident blocks than one at a time, within the shared
+    // memory of three blocks an SM
+    for (int model = 0; model < 2; ++model) {
+        const long long n = model ? p.ncg_model_blk : p.ncg_data_blk;
+        const long long room = (p.L <= 12 ? 3LL : 1LL) * num_sms;
+        int &seq = model ? p.frame_seq_model : p.frame_seq_data;
+        seq = 1;
+        for (int q = 2; q <= 4 && p.frame_pairs == 1; q *= 2) {
+            const long long rounds = ((n + q - 1) / q + room - 1) / room * q;
+            const size_t smem = frame_analysis_smem(p.L, q, model ? p.ntau : p.nt, model ? 0 : p.nt);
+            if (33 * rounds <= 34 * ((n + room - 1) / room) &&
+                smem + 1536 <= (size_t)max_smem / (p.L <= 12 ? 3 : 1))
+                seq = q;
+        }
+    }
     p.frame_ahead = (p.L <= 12 ? 3 : 1) * num_sms;       // by registers and shared memory
     const FrameFn fn = frame_pick(p.L);
     const FrameArgs none{};
@@ -73,6 +100,8 @@ cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *
     a.frac = model_side ? p.frac_s : p.frac_u;
     a.sc = FrameScatter{p.sc_i0, p.sc_n0};
     a.ahead = p.frame_pairs == 1 ? p.frame_ahead : 0;
+    // (blocked rows are whole slabs: one pair at a time)
+    a.seq = op != FRAME_R2C || blocked ? 1 : model_side ? p.frame_seq_model : p.frame_seq_data;
     a.ns = p.ns;
     a.nbins = p.nbins;
     a.tw = p.tw_t;

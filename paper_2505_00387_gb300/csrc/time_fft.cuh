@@ -51,10 +51,12 @@ struct FrameMem {
     float2 *sm;         // this pair's frame
     float2 *stg;        // this pair's staged rows, row 0 at stg
 };
+// (seq > 1: the block takes that many pairs in turn and stages all their rows.)
+__host__ __device__ constexpr int staged_rows(int nrows) { return (nrows + 6) & ~1; }
 template <class F>
-__host__ __device__ constexpr size_t frame_smem(int pairs, int nrows, int nfrac) {
+__host__ __device__ constexpr size_t frame_smem(int pairs, int seq, int nrows, int nfrac) {
     return (size_t)F::T * sizeof(float2) + (size_t)((nfrac + 3) & ~3) * sizeof(float) +
-           (size_t)pairs * (F::LEN + ((nrows + 6) & ~1)) * sizeof(float2);
+           (size_t)pairs * (F::LEN + seq * staged_rows(nrows)) * sizeof(float2);
 }
 template <class F>
 __device__ __forceinline__ FrameMem frame_mem(float4 *base, int pair, int nrows, int nfrac) {
@@ -62,8 +64,7 @@ __device__ __forceinline__ FrameMem frame_mem(float4 *base, int pair, int nrows,
     m.s_tw = reinterpret_cast<float2 *>(base);
     m.sfr = reinterpret_cast<float *>(m.s_tw + F::T);
     float2 *p = reinterpret_cast<float2 *>(m.sfr + ((nfrac + 3) & ~3));
-    const int rows = (nrows + 6) & ~1;
-    m.sm = p + (size_t)pair * (F::LEN + rows);
+    m.sm = p + (size_t)pair * (F::LEN + staged_rows(nrows));
     m.stg = m.sm + F::LEN + 1;
     return m;
 }
@@ -167,7 +168,7 @@ __device__ __forceinline__ void frame_cp(void *smem, const void *gmem) {
     if (BYTES == 16)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
     else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES));
 }
 __device__ __forceinline__ void frame_cp_wait() {
     asm volatile("cp.async.commit_group;\n");
@@ -494,6 +495,7 @@ struct FrameArgs {
     const float *__restrict__ frac;   // those fractions
     FrameScatter sc;
     int ahead;                   // blocks resident at once (0: no fetch ahead)
+    int seq;                     // pairs an analysis block takes in turn
     FistaArgs fa;
     FrameBound ybd;
 };
@@ -524,30 +526,56 @@ struct BlockPair {
     }
 };
 
-// Resample + FFT (the model's stretch S, or U^T on the data side).
+// Resample + FFT (the model's stretch S, or U^T on the data side).  A pair
+// is 8 bytes of a row of the row-major input, a quarter of the sector that
+// comes with it, so a block of one pair stages the rows of a.seq neighbouring
+// pairs together (neighbouring lanes read neighbouring pairs) and transforms
+// them in turn.
 template <class F, int INTERP, bool TRANS>
 __global__ void __launch_bounds__(F::THREADS, F::MINB)
 frame_r2c_kernel(const FrameArgs a, const float *__restrict__ in, float2 *__restrict__ out) {
     extern __shared__ float4 smem_f4[];
-    const BlockPair<F> b(a);
-    const FrameMem mem = frame_mem<F>(smem_f4, b.pair, a.nrows, a.nfrac);
-    const float *src = in + b.cg.real_off;
-    const bool two = b.cg.ncol > 1, vec = ((b.cg.real_off | b.cg.ld_real) & 1) == 0;
-    if (b.on) {
-        if (two && vec)
-            for (int r = b.t; r < a.nrows; r += F::T)
-                frame_cp<8>(mem.stg + r, src + (long long)r * b.cg.ld_real);
-        else
-            for (int r = b.t; r < a.nrows; r += F::T)
-                mem.stg[r] = row_load(src + (long long)r * b.cg.ld_real, two, false);
+    const int t = threadIdx.x % F::T, pair = threadIdx.x / F::T;
+    FrameMem mem = frame_mem<F>(smem_f4, pair, a.nrows, a.nfrac);
+    const int rows = staged_rows(a.nrows);
+    const int g0 = (blockIdx.x * (blockDim.x / F::T) + pair) * a.seq;
+    const int lseq = a.seq == 4 ? 2 : a.seq == 2 ? 1 : 0;
+    {
+        // the pair this thread stages: one of a.seq, the same in every round
+        // (T is a multiple of 4)
+        const int q = t & (a.seq - 1);
+        if (g0 + q < a.ngroups) {
+            const ColGroup cg = a.groups[g0 + q];
+            const float *src = in + cg.real_off;
+            float2 *stg = mem.stg + q * rows;
+            const bool two = cg.ncol > 1, vec = ((cg.real_off | cg.ld_real) & 1) == 0;
+            if (two && vec)
+                for (int r = t >> lseq; r < a.nrows; r += F::T >> lseq)
+                    frame_cp<8>(stg + r, src + (long long)r * cg.ld_real);
+            else               // odd row length or offset: 4-byte aligned only
+                for (int r = t >> lseq; r < a.nrows; r += F::T >> lseq) {
+                    const float *x = src + (long long)r * cg.ld_real;
+                    frame_cp<4>(&stg[r].x, x);
+                    if (two) frame_cp<4>(&stg[r].y, x + 1);
+                    else stg[r].y = 0.f;
+                }
+        }
     }
-    zero_pads(mem, a.nrows, b.t);
+    for (int q = 0; q < a.seq; ++q) {
+        const FrameMem m{mem.s_tw, mem.sfr, mem.sm, mem.stg + q * rows};
+        zero_pads(m, a.nrows, t);
+    }
     frame_tables<F>(mem.s_tw, a.tw);
     if (TRANS) copy_fractions(mem.sfr, a.frac, a.nfrac);
     frame_cp_wait();
-    __syncthreads();
-    frame_analyse<F, INTERP, TRANS>(mem, b.cg, b.on, a.ana, a.sc, a.nrows, a.tw, a.nbins, b.t,
-                                     out, a.ybd);
+    for (int q = 0; q < a.seq; ++q) {
+        __syncthreads();         // rows staged, and the last pair's frame read
+        const bool on = g0 + q < a.ngroups;
+        const ColGroup cg = a.groups[on ? g0 + q : 0];
+        frame_analyse<F, INTERP, TRANS>(mem, cg, on, a.ana, a.sc, a.nrows, a.tw, a.nbins, t, out,
+                                        a.ybd);
+        mem.stg += rows;
+    }
 }
 
 // Synthesis + resample with its epilogue: plain store, residual aux - out, or

@@ -19,8 +19,9 @@ struct FrameCall {
 template <class F, class K, class... A>
 cudaError_t frame_run(const FrameCall &c, const FrameArgs &a, int nrows, K *kern, A... args) {
     if (c.max_smem > 0) return raise_smem_limit(kern, c.max_smem);
-    const int grid = (a.ngroups + c.pairs - 1) / c.pairs;
-    kern<<<grid, F::T * c.pairs, frame_smem<F>(c.pairs, nrows, a.nfrac), c.st>>>(a, args...);
+    const int per = c.pairs * a.seq;
+    const int grid = (a.ngroups + per - 1) / per;
+    kern<<<grid, F::T * c.pairs, frame_smem<F>(c.pairs, a.seq, nrows, a.nfrac), c.st>>>(a, args...);
     return cudaGetLastError();
 }
 
