@@ -237,10 +237,11 @@ static int validate_geom(const aahrt_geom *g, int idx, bool q_explicit) {
 // run in ceil(items / resident blocks) rounds: the pair with the smallest
 // product, larger tiles (a whole warp on one trace) on a tie.
 static void choose_tiles(Plan &p, bool group_fixed, int ncube, int sms) {
-    const long long blocks = (long long)sms * (p.nos == 512 ? 1 : 3);
+    const long long blocks = (long long)sms * 3;
     double best = 1e300;
     const int given = p.tgroup;
-    for (int tile = p.nos <= 128 ? 32 : 16; tile >= 16; tile /= 2)
+    const int most = p.nos <= 128 ? 32 : p.nos == 256 ? 16 : 8, least = std::min(16, most);
+    for (int tile = most; tile >= least; tile /= 2)
         for (int ng = 1; ng <= p.ntheta; ++ng) {
             const int nj = group_fixed ? given : (p.ntheta + ng - 1) / ng;
             const long long groups = (p.ntheta + nj - 1) / nj;

@@ -59,7 +59,7 @@ template <int W_, int LR_, int TB_, int THREADS_>
 struct Tile {
     static constexpr int W = W_, LR = LR_, R = 1 << LR_, NOS = 16 << LR_, TB = TB_;
     static constexpr int THREADS = THREADS_, NSUB = THREADS_ / TB_;
-    static constexpr int MINB = THREADS_ > 256 ? 1 : 3;
+    static constexpr int MINB = 3;
     static constexpr int ROWS = NOS + W_ - 1;
 };
 
@@ -281,13 +281,14 @@ tile_fwd_kernel(const TileArgs a, const float2 *__restrict__ X, float2 *__restri
 // while spreading, and TB complex floats between the two DFT steps (every row
 // is read, rewritten and cleared by the lanes of one warp).  With TB = 16 a
 // warp spreads two traces: its halves take the real and the imaginary plane in
-// opposite order, so their rows never share a bank.
+// opposite order, so their rows never share a bank (with TB = 8, four traces:
+// pairs of them do, half the time).
 template <int TB>
 struct PlanePair {
     const int *first, *second;   // the plane this half warp takes first, and the other
     bool swap;
     __device__ __forceinline__ explicit PlanePair(const int *p)
-        : first(p), second(p + TB), swap(TB == 16 && (threadIdx.x & 16)) {
+        : first(p), second(p + TB), swap(TB < 32 && (threadIdx.x & 16)) {
         if (swap) {
             first = p + TB;
             second = p;
@@ -302,7 +303,7 @@ struct PlanePair {
 template <int TB, int W>
 __device__ __forceinline__ void tile_spread(int *G, const float *phi, int row, float vr, float vi,
                                             int bin) {
-    const bool swap = TB == 16 && (threadIdx.x & 16);
+    const bool swap = TB < 32 && (threadIdx.x & 16);
     const float x0 = swap ? vi : vr, x1 = swap ? vr : vi;
     int *p0 = G + row * 2 * TB + bin + (swap ? TB : 0);
     int *p1 = G + row * 2 * TB + bin + (swap ? 0 : TB);

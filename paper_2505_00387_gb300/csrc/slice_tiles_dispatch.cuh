@@ -3,8 +3,10 @@
 //
 // Tiles of 32 bins where two grids of nos points leave room for three blocks
 // per SM (nos <= 128), of 16 bins for 256 points (and for small plans, whose
-// work items would not fill the SMs); 512 points take one block of 512 threads
-// per SM.
+// work items would not fill the SMs), of 8 for 512 points: half the traces of a
+// pair conflict then, but three blocks share an SM (594 / 765 us forward /
+// adjoint of the 8000-trace gather against 677 / 882 with 16 bins and one block
+// of 512 threads).
 #pragma once
 
 #include "slice_tiles.cuh"
@@ -47,7 +49,7 @@ cudaError_t tile_width(const TileCall &c, const TileArgs &a, const float2 *in, f
             return wide ? tile_call<Tile<W, 3, 32, 256>>(c, a, in, out)
                         : tile_call<Tile<W, 3, 16, 256>>(c, a, in, out);
         case 256: return tile_call<Tile<W, 4, 16, 256>>(c, a, in, out);
-        case 512: return tile_call<Tile<W, 5, 16, 512>>(c, a, in, out);
+        case 512: return tile_call<Tile<W, 5, 8, 256>>(c, a, in, out);
         default: return cudaErrorInvalidValue;
     }
 }

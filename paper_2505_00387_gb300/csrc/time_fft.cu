@@ -34,7 +34,7 @@ static size_t frame_analysis_smem(int L, int seq, int nrows, int nfrac) {
 
 // Shared memory of the largest time kernel of frames of 2^L samples.
 static size_t frame_plan_smem(int L, int pairs, int nt, int ntau, int ns) {
-    const int nrows = std::max(nt, ntau), nfrac = std::max(nt, ns);
+    const int nrows = std::max(nt, ntau), nfrac = nt;
     switch (L) {
         case 9: return frame_most<2>(pairs, nrows, nfrac);
         case 10: return frame_most<4>(pairs, nrows, nfrac);
@@ -59,7 +59,8 @@ cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem) {
         p.frame_pairs /= 2;
     // pairs an analysis block of one pair takes in turn: as many as cost at most
     // 3 % more rounds of resident blocks than one at a time, within the shared
-    // memory of three blocks an SM
+    // memory of three blocks an SM (10 % where a block has its SM to itself
+    // and nothing else hides the wait for its rows)
     for (int model = 0; model < 2; ++model) {
         const long long n = model ? p.ncg_model_blk : p.ncg_data_blk;
         const long long room = (p.L <= 12 ? 3LL : 1LL) * num_sms;
@@ -68,12 +69,12 @@ cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem) {
         for (int q = 2; q <= 4 && p.frame_pairs == 1; q *= 2) {
             const long long rounds = ((n + q - 1) / q + room - 1) / room * q;
             const size_t smem = frame_analysis_smem(p.L, q, model ? p.ntau : p.nt, model ? 0 : p.nt);
-            if (33 * rounds <= 34 * ((n + room - 1) / room) &&
+            if (100 * rounds <= (p.L <= 12 ? 103 : 110) * ((n + room - 1) / room) &&
                 smem + 1536 <= (size_t)max_smem / (p.L <= 12 ? 3 : 1))
                 seq = q;
         }
     }
-    p.frame_ahead = (p.L <= 12 ? 3 : 1) * num_sms;       // by registers and shared memory
+    p.frame_ahead = (p.L <= 12 ? 4 : 2) * num_sms;       // resident blocks, by registers
     const FrameFn fn = frame_pick(p.L);
     const FrameArgs none{};
     cudaError_t e = cudaSuccess;
@@ -95,8 +96,8 @@ cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *
     a.syn = model_side ? p.ST : p.U;
     a.ana = model_side ? p.S : p.UT;
     a.nrows = model_side ? p.ntau : p.nt;
-    // fractions: of S^T in a model synthesis, of U^T in a data analysis
-    a.nfrac = model_side ? (op == FRAME_R2C ? 0 : p.ns) : (op == FRAME_C2R ? 0 : p.nt);
+    // fractions staged: those of U^T, in a data analysis
+    a.nfrac = model_side || op == FRAME_C2R ? 0 : p.nt;
     a.frac = model_side ? p.frac_s : p.frac_u;
     a.sc = FrameScatter{p.sc_i0, p.sc_n0};
     a.ahead = p.frame_pairs == 1 ? p.frame_ahead : 0;

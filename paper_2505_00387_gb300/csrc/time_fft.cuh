@@ -37,7 +37,10 @@ struct Frame {
     // exchange or natural frame with one zero sample either side
     static constexpr int LEN = N + N / 16 + 4;
     static constexpr int THREADS = T > 256 ? T : 256;  // most threads of a block
-    static constexpr int MINB = T > 256 ? 1 : 3;
+    // blocks an SM holds: four (two of 512 threads) at 64 registers; the
+    // analysis alone keeps 80, which its table entries and rows in flight need
+    // (430 against 535 us for the model columns of 32 cubes)
+    static constexpr int MINB = T > 256 ? 2 : 4, MINB_ANA = T > 256 ? 1 : 3;
 };
 
 __device__ __forceinline__ int frame_at(int n) { return 2 + n + (n >> 4); }
@@ -440,7 +443,8 @@ __device__ __forceinline__ int2 frame_entry(const DevResampler &rs, int i) {
                                                       : (const void *)(rs.pos + i)));
 }
 template <int INTERP, bool TRANS>
-__device__ __forceinline__ float2 frame_row(const FrameMem &mem, int2 e) {
+__device__ __forceinline__ float2 frame_row(const FrameMem &mem, const float *__restrict__ frac,
+                                            int2 e) {
     float2 s = make_float2(0.f, 0.f);
     if (!TRANS) {
         const float fr = __int_as_float(e.y);
@@ -458,7 +462,7 @@ __device__ __forceinline__ float2 frame_row(const FrameMem &mem, int2 e) {
         for (int q = Taps<INTERP>::n - 1; q >= 0; --q) {
             const int cnt = (e.y >> (8 * q)) & 255;
             for (int j = 0; j < cnt; ++j, ++r) {
-                const float w = tap_weight<INTERP>(Taps<INTERP>::t0 + q, mem.sfr[r]);
+                const float w = tap_weight<INTERP>(Taps<INTERP>::t0 + q, __ldg(frac + r));
                 const float2 x = mem.sm[frame_at(r)];
                 s.x = fmaf(w, x.x, s.x);
                 s.y = fmaf(w, x.y, s.y);
@@ -532,7 +536,7 @@ struct BlockPair {
 // pairs together (neighbouring lanes read neighbouring pairs) and transforms
 // them in turn.
 template <class F, int INTERP, bool TRANS>
-__global__ void __launch_bounds__(F::THREADS, F::MINB)
+__global__ void __launch_bounds__(F::THREADS, F::MINB_ANA)
 frame_r2c_kernel(const FrameArgs a, const float *__restrict__ in, float2 *__restrict__ out) {
     extern __shared__ float4 smem_f4[];
     const int t = threadIdx.x % F::T, pair = threadIdx.x / F::T;
@@ -588,7 +592,6 @@ frame_c2r_kernel(const FrameArgs a, const float2 *__restrict__ in, float *__rest
     const BlockPair<F> b(a);
     const FrameMem mem = frame_mem<F>(smem_f4, b.pair, 0, a.nfrac);
     frame_fetch<F>(mem, b.cg, b.on, in, a.nbins, b.t);
-    if (TRANS) copy_fractions(mem.sfr, a.frac, a.nfrac);
     frame_tables<F>(mem.s_tw, a.tw);
     if (threadIdx.x == 0 && a.ahead > 0 && blockIdx.x + a.ahead < gridDim.x)
         prefetch_l2(in + a.groups[blockIdx.x + a.ahead].bins_off,
@@ -610,7 +613,7 @@ frame_c2r_kernel(const FrameArgs a, const float2 *__restrict__ in, float *__rest
             x = row_load(a.fa.m + o, two, vec);
             z = row_load(a.fa.z + o, two, vec);
         }
-        const float2 g = frame_row<INTERP, TRANS>(mem, e);
+        const float2 g = frame_row<INTERP, TRANS>(mem, a.frac, e);
         if (EPI == EPI_STORE) {
             row_store(out + o, g, two, vec);
         } else if (EPI == EPI_RESIDUAL) {
@@ -641,7 +644,7 @@ frame_fused_kernel(const FrameArgs a, float2 *spec, const float *__restrict__ au
         reinterpret_cast<const float2 *>((EPI == EPI_RESIDUAL ? aux : a.fa.z) + b.cg.real_off);
     if (b.on)
         for (int i = b.t; i < a.nrows; i += F::T) frame_cp<8>(mem.stg + i, state + i);
-    copy_fractions(mem.sfr, a.frac, a.nfrac);
+    if (!SYN_TRANS) copy_fractions(mem.sfr, a.frac, a.nfrac);
     frame_tables<F>(mem.s_tw, a.tw);
     zero_pads(mem, a.nrows, b.t);
     if (threadIdx.x < 3 && a.ahead > 0 && blockIdx.x + a.ahead < gridDim.x) {
@@ -667,7 +670,7 @@ frame_fused_kernel(const FrameArgs a, float2 *spec, const float *__restrict__ au
         const float2 m = mnxt;
         nxt = frame_entry<SYN_TRANS>(a.syn, min(i + F::T, last));
         if (EPI == EPI_FISTA) mnxt = mrow[min(i + F::T, last)];
-        const float2 g = frame_row<INTERP, SYN_TRANS>(mem, e);
+        const float2 g = frame_row<INTERP, SYN_TRANS>(mem, a.frac, e);
         const float2 s = mem.stg[i];
         float2 x;
         if (EPI == EPI_RESIDUAL) {
