@@ -39,8 +39,8 @@ struct EsPoly {
 
 struct TapSet {
     int u0;      // first grid point (may be negative; index mod nos)
-    float g;     // centred offset of the position, [-1/2, 1/2)
-    float ph;    // phase in cycles, [-1/2, 1/2)
+    float g;     // centred offset of the position, [-1/2, 1/2]
+    float ph;    // phase in cycles, [-1/2, 1/2]
 };
 
 template <int W>
@@ -54,14 +54,15 @@ __host__ __device__ __forceinline__ TapSet trace_taps(unsigned long long A,
     TapSet t;
     t.ph = (float)(int)ptop * 2.3283064365386963e-10f;      // 2^-32
     const int iu = (int)(xtop >> (32 - Lq));                  // integer part of nos*x
-    const float fy = (float)(unsigned)(xtop << Lq) * 2.3283064365386963e-10f;
+    // the fraction as a signed word: odd W centres it on the nearest grid point
+    // (fractions from 1/2 up belong to the next one), even W on the half
+    const unsigned fr = xtop << Lq;
     if (W & 1) {
-        const bool up = fy >= 0.5f;
-        t.u0 = iu - (W - 1) / 2 + (up ? 1 : 0);
-        t.g = up ? fy - 1.0f : fy;
+        t.u0 = iu - (W - 1) / 2 + (int)(fr >> 31);
+        t.g = (float)(int)fr * 2.3283064365386963e-10f;       // 2^-32
     } else {
         t.u0 = iu - W / 2 + 1;
-        t.g = fy - 0.5f;
+        t.g = (float)(int)(fr ^ 0x80000000u) * 2.3283064365386963e-10f;
     }
     return t;
 }

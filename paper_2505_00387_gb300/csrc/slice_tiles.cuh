@@ -64,13 +64,14 @@ struct Tile {
 };
 
 // s_tw[16 n2 + p1] = exp(-2 pi i n2 p1 / nos), the twiddles between the two
-// steps; s_dec[u] = factor of curvature l = (u + cq) mod nos (0 beyond nq).
+// steps; s_dec[u] = factor of curvature l = (u + cq) mod nos (0 beyond nq),
+// with the operator's 1/Nfft (a power of two, so it changes no rounding).
 template <class T>
 __device__ __forceinline__ void tile_tables(const TileArgs &a, float2 *s_tw, float *s_dec) {
     for (int i = threadIdx.x; i < T::NOS; i += T::THREADS) {
         s_tw[i] = __ldg(a.tw + (i >> 4) * (i & 15));
         const int l = (i + a.cq) & (T::NOS - 1);
-        s_dec[i] = l < a.nq ? __ldg(a.dec + l) : 0.f;
+        s_dec[i] = l < a.nq ? a.scale * __ldg(a.dec + l) : 0.f;
     }
 }
 
@@ -265,7 +266,7 @@ tile_fwd_kernel(const TileArgs a, const float2 *__restrict__ X, float2 *__restri
                 // times exp(-2 pi i ph) = cs - i sn
                 if (live)
                     Yc[(long long)tr.col * a.nbins] =
-                        make_float2(a.scale * (ar * cs + ai * sn), a.scale * (ai * cs - ar * sn));
+                        make_float2(ar * cs + ai * sn, ai * cs - ar * sn);
             }
             __syncthreads();
             cur ^= 1;
@@ -447,7 +448,7 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
             const int jn = j + 1 == a.ntheta ? 0 : j + 1;
             const int t0 = ss[j], t1 = ss[j + 1];
             const float bound0 = bound1;
-            bound1 = M * __ldg(ws + jn) * a.scale * a.phicap;
+            bound1 = M * __ldg(ws + jn) * a.phicap;
             const float fx0 = bound0 > 0.f ? 1073741824.0f / bound0 : 0.f;   // 2^30 / bound
             const float fx1 = bound1 > 0.f ? 1073741824.0f / bound1 : 0.f;
             const bool own0 = jj >= 0, own1 = jj + 1 < g.nj;
@@ -470,9 +471,9 @@ tile_adj_kernel(const TileArgs a, const float2 *__restrict__ Y, float2 *__restri
                     es_weights<W>(a.poly, ts.g, phi);
                     float sn, cs;
                     phase_cs(ts.ph, &sn, &cs);
-                    // scale * y * exp(+2 pi i ph)
-                    const float vr = a.scale * (y.x * cs - y.y * sn);
-                    const float vi = a.scale * (y.x * sn + y.y * cs);
+                    // y * exp(+2 pi i ph)
+                    const float vr = y.x * cs - y.y * sn;
+                    const float vi = y.x * sn + y.y * cs;
                     const int row = ts.u0 & (T::NOS - 1);
                     const float f0 = tr.w0 * fx0, f1 = tr.w1 * fx1;
                     if (own0) tile_spread<TB, W>(G0, phi, row, f0 * vr, f0 * vi, bin);
