@@ -107,7 +107,8 @@ cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *
     a.nbins = p.nbins;
     a.tw = p.tw_t;
     a.fa = fa;
-    a.ybd = bound ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
+    // (the direct sum has no fixed point, so no bound to keep)
+    a.ybd = bound && p.slice_interp != AAHRT_SLICE_DIRECT ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
     return frame_pick(p.L)(FrameCall{(FrameOp)op, model_side, p.interp, epi, p.frame_pairs, st, 0}, a,
                            in, out, aux);
 }
