@@ -22,7 +22,7 @@
 //   A B ~ A_hi B_hi + A_hi B_lo + A_lo B_hi   (FP32 accumulation in TMEM).
 // The phase arguments are range-reduced exactly in 64-bit fixed point.
 //
-// One CTA of 16 warps per SM (persistent), warp-specialized: producer warps
+// One CTA of 21 warps per SM (persistent), warp-specialized: producer warps
 // build the bf16 operand tiles of each K chunk (64 K-elements) in shared
 // memory (128-byte swizzled K-major layout) into a ring of two stages, one
 // thread issues the MMAs and commits each stage back to the producers through
@@ -37,7 +37,7 @@ namespace aahrt {
 
 using namespace tc;
 
-constexpr int kTcThreads = 512;
+constexpr int kTcThreads = 672;
 constexpr uint32_t kTileA = 128u * 128u;     // one 128-row x 64-element bf16 tile
 constexpr uint32_t kTcWait = 1u << 24;       // mbarrier polls before giving up
 constexpr int kTcMaxGp = 64;
@@ -119,16 +119,13 @@ __device__ __forceinline__ float2 cmul2(float2 a, float2 b) {
 }
 
 // Eight consecutive q samples l0 .. l0+7 of exp(sgn 2 pi i f_k q_l r^2) (zero
-// for l >= nq): the phase of l is k*A + (l - cq)*k*B in fixed point.
-__device__ __forceinline__ void phases8(const TraceGeo &tr, unsigned k, int l0, int cq, int nq,
-                                        float sgn, float wgt, float2 *e) {
-    const unsigned long long kb = (unsigned long long)k * tr.B;
-    const unsigned long long p0 =
-        (unsigned long long)k * tr.A + (unsigned long long)(long long)(l0 - cq) * kb;
-    float2 z = cis_fixed(p0, sgn);
+// for l >= nq): the phase of l is ka + (l - cq) kb in fixed point, ka = k A,
+// kb = k B; st = exp(sgn 2 pi i kb).
+__device__ __forceinline__ void phases8(unsigned long long ka, unsigned long long kb, float2 st,
+                                        int l0, int cq, int nq, float sgn, float wgt, float2 *e) {
+    float2 z = cis_fixed(ka + (unsigned long long)(long long)(l0 - cq) * kb, sgn);
     z.x *= wgt;
     z.y *= wgt;
-    const float2 st = cis_fixed(kb, sgn);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         e[i] = l0 + i < nq ? z : make_float2(0.f, 0.f);
@@ -137,12 +134,10 @@ __device__ __forceinline__ void phases8(const TraceGeo &tr, unsigned k, int l0, 
 }
 
 // The same eight samples on an explicit (non-uniform) curvature axis: the
-// phase of l is k*A + qn[l]*k*B, one rotation per sample.
-__device__ __forceinline__ void phases8_axis(const TraceGeo &tr, unsigned k, int l0,
+// phase of l is ka + qn[l] kb, one rotation per sample.
+__device__ __forceinline__ void phases8_axis(unsigned long long ka, unsigned long long kb, int l0,
                                              const long long *qn, int nq, float sgn, float wgt,
                                              float2 *e) {
-    const unsigned long long ka = (unsigned long long)k * tr.A;
-    const unsigned long long kb = (unsigned long long)k * tr.B;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int l = l0 + i;
@@ -155,12 +150,27 @@ __device__ __forceinline__ void phases8_axis(const TraceGeo &tr, unsigned k, int
     }
 }
 
+// Gathers g and g + 1 (g even) of a row of G: one 16-byte store where G is even
+// (rows then start at 16-byte boundaries).
+__device__ __forceinline__ void store_gathers(float2 *row, int g, int G, float4 v) {
+    if ((G & 1) == 0) {
+        if (g < G) *reinterpret_cast<float4 *>(row + g) = v;
+    } else {
+        if (g < G) row[g] = make_float2(v.x, v.y);
+        if (g + 1 < G) row[g + 1] = make_float2(v.z, v.w);
+    }
+}
+
 // ------------------------------------------------------ pipeline roles
-// Warp 0 allocates the TMEM (two accumulator buffers of 256 columns) and
-// its lane 0 issues the MMAs; warps 1..11 build the operand tiles into a
-// ring of two shared-memory stages; warps 12..15 (one per TMEM lane quarter)
-// drain a finished accumulator to global memory while the tensor core fills
-// the other.  Four kinds of mbarrier hand the stages and accumulators
+// Warps 0..3 (one per TMEM lane quarter) drain a finished accumulator to
+// global memory while the tensor core fills the other; warp 4 allocates the
+// TMEM (two accumulator buffers of 256 columns) and its lane 0 issues the MMAs;
+// warps 5..20 build the operand tiles into a ring of two shared-memory stages.
+// The producers pace the kernel (instructions, and latency of the operand
+// loads), so there are as many as 96 registers a thread allow, and with 64
+// gathers each thread's share of a K chunk is whole: one A and one B unit
+// (forward), two and one (adjoint).  The B operands of a chunk, and the
+// adjoint's trace, are loaded before the wait for a free stage.  Four kinds of mbarrier hand the stages and accumulators
 // around:
 //   full[s]   producers -> MMA    (stage s written; one arrival per producer thread)
 //   empty[s]  MMA -> producers    (tcgen05.commit: the MMAs reading stage s are done)
@@ -171,10 +181,10 @@ __device__ __forceinline__ void phases8_axis(const TraceGeo &tr, unsigned k, int
 // wait that runs out sets the error flag and the block's abort flag, which
 // ends every role's loop, and the MMA thread waits (bounded) for its last
 // commit before the TMEM is released.
-constexpr int kTcProdWarp0 = 1;
-constexpr int kTcProdWarps = 11;
-constexpr int kTcProdThreads = 32 * kTcProdWarps;
-constexpr int kTcEpiWarp0 = 12;          // warps 12..15: TMEM lane quarters 0..3
+constexpr int kTcMmaWarp = 4;            // warps 0..3: TMEM lane quarters 0..3
+constexpr int kTcProdWarp0 = 5;
+constexpr int kTcProdThreads = kTcThreads - 32 * kTcProdWarp0;
+static_assert(kTcProdThreads == 512, "one A unit (forward) or one trace lane per producer");
 constexpr uint32_t kTcTmemCols = 512;    // two accumulators of 256 columns
 
 struct TcBars {
@@ -183,7 +193,7 @@ struct TcBars {
 
 __device__ __forceinline__ void tc_setup(TcBars *bars, uint32_t *tmem_slot, int *abort) {
     const int warp = threadIdx.x >> 5;
-    if (warp == 0) tmem_alloc(smem_u32(tmem_slot), kTcTmemCols);
+    if (warp == kTcMmaWarp) tmem_alloc(smem_u32(tmem_slot), kTcTmemCols);
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&bars->full[i]), kTcProdThreads);
@@ -234,7 +244,7 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
     tc_setup(&bars, &tmem_slot, &s_abort);
     const uint32_t tm = tmem_slot;
 
-    if (warp == 0) {
+    if (warp == kTcMmaWarp) {
         // ---------------------------------------------------------- MMA
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16_f32(128, N);
@@ -281,7 +291,7 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
             // the TMEM is released only after the MMAs issued have finished
             if (issued) mbar_wait(last_bar, last_par, kTcWait, a.wait_ns);
         }
-    } else if (warp < kTcEpiWarp0) {
+    } else if (warp >= kTcProdWarp0) {
         // ---------------------------------------------------- producers
         const int pid = tid - 32 * kTcProdWarp0;
         const float inv_gp = 1.0f / (float)Gp;
@@ -294,62 +304,69 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
             const long long blk = (long long)a.nq * a.G;      // one (bin, slice) block of X
             const float2 *Xj = X + ((long long)j * a.nbins + k) * blk;
             const float2 *Xn = X + ((long long)jn * a.nbins + k) * blk;
+            // A unit: trace r of the tile, 8 q samples; its phase per q step is
+            // the same in every chunk
+            const int r = pid >> 2, lb = pid & 3;
+            const bool trace = t0 + r < t1;
+            unsigned long long ka = 0, kb = 0;
+            if (trace) {
+                const TraceGeo *tr = a.geo + t0 + r;
+                ka = (unsigned long long)k * tr->A;
+                kb = (unsigned long long)k * tr->B;
+            }
+            const float2 st8 = cis_fixed(kb, -1.f);
+            // B unit: slice sl, gather g, 8 q samples
+            const int rest = tc_div(pid, Gp, inv_gp);
+            const int g = pid - rest * Gp, sl = rest & 1, lbb = rest >> 1;
+            const bool col = pid < 8 * Gp;
+            const float2 *Xs = (sl ? Xn : Xj) + g;
             for (int c = 0; c < nch; ++c, ++cc) {
+                float2 x[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int l = 32 * c + 8 * lbb + i;
+                    x[i] = make_float2(0.f, 0.f);
+                    if (col && l < a.nq && g < a.G) x[i] = __ldg(Xs + (long long)l * a.G);
+                }
                 const int st = cc & 1;
                 if (!tc_wait_bar(a, &bars.empty[st], ((cc >> 1) & 1) ^ 1, abort)) break;
                 unsigned char *ahi = sm + st * stage_bytes, *alo = ahi + kTileA;
                 unsigned char *bhi = alo + kTileA, *blo = bhi + bbytes;
-                for (int u = pid; u < 128 * 4 + 8 * Gp; u += kTcProdThreads) {
-                    if (u < 128 * 4) {
-                        // A: E[h][l] for 128 traces x 32 q samples, (Re, Im) interleaved
-                        const int r = u >> 2, lb = u & 3;
-                        const int t = t0 + r;
-                        float2 e[8];
-                        if (t < t1) {
-                            const TraceGeo tr = a.geo[t];
-                            if (a.qn)
-                                phases8_axis(tr, (unsigned)k, 32 * c + 8 * lb, a.qn, a.nq, -1.f,
-                                             1.f, e);
-                            else
-                                phases8(tr, (unsigned)k, 32 * c + 8 * lb, a.cq, a.nq, -1.f, 1.f,
-                                        e);
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) e[i] = make_float2(0.f, 0.f);
-                        }
-                        uint4 h0, l0, h1, l1;
-                        split8(reinterpret_cast<const float *>(e), &h0, &l0);
-                        split8(reinterpret_cast<const float *>(e) + 8, &h1, &l1);
-                        st_chunk(ahi, r, 2 * lb, h0);
-                        st_chunk(ahi, r, 2 * lb + 1, h1);
-                        st_chunk(alo, r, 2 * lb, l0);
-                        st_chunk(alo, r, 2 * lb + 1, l1);
+                {
+                    // A: E[h][l] for 128 traces x 32 q samples, (Re, Im) interleaved
+                    float2 e[8];
+                    if (trace) {
+                        if (a.qn)
+                            phases8_axis(ka, kb, 32 * c + 8 * lb, a.qn, a.nq, -1.f, 1.f, e);
+                        else
+                            phases8(ka, kb, st8, 32 * c + 8 * lb, a.cq, a.nq, -1.f, 1.f, e);
                     } else {
-                        // B: rows (part, slice, g), K = the chunk's q samples
-                        const int v = u - 128 * 4;
-                        const int rest = tc_div(v, Gp, inv_gp);
-                        const int g = v - rest * Gp;
-                        const int sl = rest & 1, lb = rest >> 1;
-                        const float2 *Xs = sl ? Xn : Xj;
-                        const int l0 = 32 * c + 8 * lb;
-                        uint32_t rh[8], rl[8], ih[8], il[8];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int l = l0 + i;
-                            float2 x = make_float2(0.f, 0.f);
-                            if (l < a.nq && g < a.G) x = __ldg(Xs + (long long)l * a.G + g);
-                            split_cplx(x.x, x.y, &rh[i], &rl[i], &ih[i], &il[i]);
-                        }
-                        const int nre = sl * Gp + g, nim = 2 * Gp + sl * Gp + g;
-                        st_chunk(bhi, nre, 2 * lb, make_uint4(rh[0], rh[1], rh[2], rh[3]));
-                        st_chunk(bhi, nre, 2 * lb + 1, make_uint4(rh[4], rh[5], rh[6], rh[7]));
-                        st_chunk(blo, nre, 2 * lb, make_uint4(rl[0], rl[1], rl[2], rl[3]));
-                        st_chunk(blo, nre, 2 * lb + 1, make_uint4(rl[4], rl[5], rl[6], rl[7]));
-                        st_chunk(bhi, nim, 2 * lb, make_uint4(ih[0], ih[1], ih[2], ih[3]));
-                        st_chunk(bhi, nim, 2 * lb + 1, make_uint4(ih[4], ih[5], ih[6], ih[7]));
-                        st_chunk(blo, nim, 2 * lb, make_uint4(il[0], il[1], il[2], il[3]));
-                        st_chunk(blo, nim, 2 * lb + 1, make_uint4(il[4], il[5], il[6], il[7]));
+                        for (int i = 0; i < 8; ++i) e[i] = make_float2(0.f, 0.f);
                     }
+                    uint4 h0, l0, h1, l1;
+                    split8(reinterpret_cast<const float *>(e), &h0, &l0);
+                    split8(reinterpret_cast<const float *>(e) + 8, &h1, &l1);
+                    st_chunk(ahi, r, 2 * lb, h0);
+                    st_chunk(ahi, r, 2 * lb + 1, h1);
+                    st_chunk(alo, r, 2 * lb, l0);
+                    st_chunk(alo, r, 2 * lb + 1, l1);
+                }
+                if (col) {
+                    // B: rows (part, slice, g), K = the chunk's q samples
+                    uint32_t rh[8], rl[8], ih[8], il[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        split_cplx(x[i].x, x[i].y, &rh[i], &rl[i], &ih[i], &il[i]);
+                    const int nre = sl * Gp + g, nim = 2 * Gp + sl * Gp + g;
+                    st_chunk(bhi, nre, 2 * lbb, make_uint4(rh[0], rh[1], rh[2], rh[3]));
+                    st_chunk(bhi, nre, 2 * lbb + 1, make_uint4(rh[4], rh[5], rh[6], rh[7]));
+                    st_chunk(blo, nre, 2 * lbb, make_uint4(rl[0], rl[1], rl[2], rl[3]));
+                    st_chunk(blo, nre, 2 * lbb + 1, make_uint4(rl[4], rl[5], rl[6], rl[7]));
+                    st_chunk(bhi, nim, 2 * lbb, make_uint4(ih[0], ih[1], ih[2], ih[3]));
+                    st_chunk(bhi, nim, 2 * lbb + 1, make_uint4(ih[4], ih[5], ih[6], ih[7]));
+                    st_chunk(blo, nim, 2 * lbb, make_uint4(il[0], il[1], il[2], il[3]));
+                    st_chunk(blo, nim, 2 * lbb + 1, make_uint4(il[4], il[5], il[6], il[7]));
                 }
                 fence_async_smem();     // this thread's tile writes -> the tensor core
                 mbar_arrive(smem_u32(&bars.full[st]));
@@ -385,10 +402,12 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
                 tmem_ld16(lanebase + 3 * Gp + gb, im1);
                 if (valid) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (gb + i < a.G)
-                            Yrow[gb + i] = make_float2(fmaf(w0, re0[i], w1 * re1[i]),
-                                                       fmaf(w0, im0[i], w1 * im1[i]));
+                    for (int i = 0; i < 16; i += 2)
+                        store_gathers(Yrow, gb + i, a.G,
+                                      make_float4(fmaf(w0, re0[i], w1 * re1[i]),
+                                                  fmaf(w0, im0[i], w1 * im1[i]),
+                                                  fmaf(w0, re0[i + 1], w1 * re1[i + 1]),
+                                                  fmaf(w0, im0[i + 1], w1 * im1[i + 1])));
                 }
             }
             fence_before_sync();
@@ -398,7 +417,7 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
     }
     fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTcTmemCols);
+    if (warp == kTcMmaWarp) tmem_dealloc(tm, kTcTmemCols);
 }
 
 // ------------------------------------------------------------- adjoint
@@ -423,7 +442,7 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
     tc_setup(&bars, &tmem_slot, &s_abort);
     const uint32_t tm = tmem_slot;
 
-    if (warp == 0) {
+    if (warp == kTcMmaWarp) {
         // ---------------------------------------------------------- MMA
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16_f32(128, N);
@@ -479,11 +498,10 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
             }
             if (issued) mbar_wait(last_bar, last_par, kTcWait, a.wait_ns);
         }
-    } else if (warp < kTcEpiWarp0) {
+    } else if (warp >= kTcProdWarp0) {
         // ---------------------------------------------------- producers
         const int pid = tid - 32 * kTcProdWarp0;
         const float inv_gp = 1.0f / (float)Gp;
-        const int na = 32 * 16 * nmt;    // A units: (trace, 8-q group)
         uint32_t cc = 0;
         for (long long item = blockIdx.x; item < a.total && !*abort; item += gridDim.x) {
             const int k = (int)(item / J);
@@ -495,61 +513,69 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
             const int nch = (ntot + 31) >> 5;
             const float2 *Ya = Yh + ((long long)a.nbins * a0 + (long long)k * n1) * a.G;
             const float2 *Yb = Yh + ((long long)a.nbins * b0 + (long long)k * n2) * a.G;
+            // A units: trace lane hh of the chunk, 8 q samples (one unit per M
+            // tile); B unit: gather g, 4 traces (a 16-byte chunk of a row pair)
+            const int hh = pid & 31;
+            const int tq = tc_div(pid, Gp, inv_gp);
+            const int g = pid - tq * Gp;
+            const bool col = pid < 8 * Gp;
             for (int c = 0; c < nch; ++c, ++cc) {
+                const int p = 32 * c + hh;
+                unsigned long long ka = 0, kb = 0;
+                float wgt = 0.f;
+                if (p < ntot) {
+                    const TraceGeo tr = a.geo[p < n1 ? a0 + p : b0 + (p - n1)];
+                    ka = (unsigned long long)k * tr.A;
+                    kb = (unsigned long long)k * tr.B;
+                    wgt = p < n1 ? tr.w0 : tr.w1;
+                }
+                float2 y[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int py = 32 * c + 4 * tq + i;
+                    y[i] = make_float2(0.f, 0.f);
+                    if (col && py < ntot && g < a.G)
+                        y[i] = __ldg(py < n1 ? Ya + (long long)py * a.G + g
+                                             : Yb + (long long)(py - n1) * a.G + g);
+                }
                 const int st = cc & 1;
                 if (!tc_wait_bar(a, &bars.empty[st], ((cc >> 1) & 1) ^ 1, abort)) break;
                 unsigned char *st0 = sm + st * stage_bytes;
                 unsigned char *bhi = st0 + 4 * kTileA, *blo = bhi + bbytes;
-                for (int u = pid; u < na + 8 * Gp; u += kTcProdThreads) {
-                    if (u < na) {
-                        // A: w conj(E)[l][h], rows l (M tiles), K = 32 traces
-                        const int hh = u & 31, lb = u >> 5;
-                        const int p = 32 * c + hh;
-                        const int l0 = 8 * lb;
-                        const int mt = l0 >> 7;
-                        unsigned char *ahi = st0 + (2 * mt) * kTileA, *alo = ahi + kTileA;
-                        float2 e[8];
-                        if (p < ntot) {
-                            const TraceGeo tr = a.geo[p < n1 ? a0 + p : b0 + (p - n1)];
-                            const float wgt = p < n1 ? tr.w0 : tr.w1;
-                            if (a.qn)
-                                phases8_axis(tr, (unsigned)k, l0, a.qn, a.nq, 1.f, wgt, e);
-                            else
-                                phases8(tr, (unsigned)k, l0, a.cq, a.nq, 1.f, wgt, e);
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) e[i] = make_float2(0.f, 0.f);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int r = (l0 & 127) + i;
-                            uint32_t h, lo;
-                            split2(e[i].x, e[i].y, &h, &lo);
-                            const uint32_t off = sw128_offset((uint32_t)r, (uint32_t)(2 * hh));
-                            *reinterpret_cast<uint32_t *>(ahi + off) = h;
-                            *reinterpret_cast<uint32_t *>(alo + off) = lo;
-                        }
+                const float2 st8 = cis_fixed(kb, 1.f);
+                for (int mt = 0; mt < nmt; ++mt) {
+                    // A: w conj(E)[l][h], rows l of the M tile, K = 32 traces
+                    const int lr = 8 * (pid >> 5), l0 = 128 * mt + lr;
+                    unsigned char *ahi = st0 + (2 * mt) * kTileA, *alo = ahi + kTileA;
+                    float2 e[8];
+                    if (p < ntot) {
+                        if (a.qn)
+                            phases8_axis(ka, kb, l0, a.qn, a.nq, 1.f, wgt, e);
+                        else
+                            phases8(ka, kb, st8, l0, a.cq, a.nq, 1.f, wgt, e);
                     } else {
-                        // B: rows (part, g), K = 32 traces x (Re, Im); one unit is
-                        // one 16-byte chunk (4 traces) of a row pair
-                        const int v = u - na;
-                        const int tq = tc_div(v, Gp, inv_gp);
-                        const int g = v - tq * Gp;
-                        uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int p = 32 * c + 4 * tq + i;
-                            float2 y = make_float2(0.f, 0.f);
-                            if (p < ntot && g < a.G)
-                                y = __ldg(p < n1 ? Ya + (long long)p * a.G + g
-                                                 : Yb + (long long)(p - n1) * a.G + g);
-                            split_cplx(y.x, y.y, &rh[i], &rl[i], &ih[i], &il[i]);
-                        }
-                        st_chunk(bhi, g, tq, make_uint4(rh[0], rh[1], rh[2], rh[3]));
-                        st_chunk(blo, g, tq, make_uint4(rl[0], rl[1], rl[2], rl[3]));
-                        st_chunk(bhi, Gp + g, tq, make_uint4(ih[0], ih[1], ih[2], ih[3]));
-                        st_chunk(blo, Gp + g, tq, make_uint4(il[0], il[1], il[2], il[3]));
+                        for (int i = 0; i < 8; ++i) e[i] = make_float2(0.f, 0.f);
                     }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        uint32_t h, lo;
+                        split2(e[i].x, e[i].y, &h, &lo);
+                        const uint32_t off = sw128_offset((uint32_t)(lr + i), (uint32_t)(2 * hh));
+                        *reinterpret_cast<uint32_t *>(ahi + off) = h;
+                        *reinterpret_cast<uint32_t *>(alo + off) = lo;
+                    }
+                }
+                if (col) {
+                    // B: rows (part, g), K = 32 traces x (Re, Im)
+                    uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        split_cplx(y[i].x, y[i].y, &rh[i], &rl[i], &ih[i], &il[i]);
+                    st_chunk(bhi, g, tq, make_uint4(rh[0], rh[1], rh[2], rh[3]));
+                    st_chunk(blo, g, tq, make_uint4(rl[0], rl[1], rl[2], rl[3]));
+                    st_chunk(bhi, Gp + g, tq, make_uint4(ih[0], ih[1], ih[2], ih[3]));
+                    st_chunk(blo, Gp + g, tq, make_uint4(il[0], il[1], il[2], il[3]));
                 }
                 fence_async_smem();
                 mbar_arrive(smem_u32(&bars.full[st]));
@@ -585,9 +611,10 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
                     }
                     if (l < a.nq) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            if (gb + i < a.G)
-                                Xrow[gb + i] = make_float2(a.scale * re[i], a.scale * im[i]);
+                        for (int i = 0; i < 16; i += 2)
+                            store_gathers(Xrow, gb + i, a.G,
+                                          make_float4(a.scale * re[i], a.scale * im[i],
+                                                      a.scale * re[i + 1], a.scale * im[i + 1]));
                     }
                 }
             }
@@ -598,7 +625,7 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
     }
     fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTcTmemCols);
+    if (warp == kTcMmaWarp) tmem_dealloc(tm, kTcTmemCols);
 }
 
 // ------------------------------------------------------------- host side
