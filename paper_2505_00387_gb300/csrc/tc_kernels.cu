@@ -53,6 +53,7 @@ struct TcArgs {
     unsigned long long wait_ns;           // device time a wait may take before giving up
     int stall;                            // test hook: issue no matrix operations
     int ntiles, nbins, nq, ntheta, G, Gp, ntr, cq;
+    int wide;                             // output rows start at 32-byte sectors
     float scale;
 };
 
@@ -150,14 +151,24 @@ __device__ __forceinline__ void phases8_axis(unsigned long long ka, unsigned lon
     }
 }
 
-// Gathers g and g + 1 (g even) of a row of G: one 16-byte store where G is even
-// (rows then start at 16-byte boundaries).
-__device__ __forceinline__ void store_gathers(float2 *row, int g, int G, float4 v) {
-    if ((G & 1) == 0) {
-        if (g < G) *reinterpret_cast<float4 *>(row + g) = v;
+// Gathers g .. g + 3 (g a multiple of 4) of a row of G, v = (re, im) of each:
+// one 32-byte sector a store where rows start at sectors (wide: G a multiple of
+// 4, the spectrum 32-byte aligned), 16-byte stores for an even G.
+__device__ __forceinline__ void store_gathers(float2 *row, int g, int G, int wide,
+                                              const float2 *v) {
+    if (wide) {
+        if (g < G)
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(row + g),
+                         "f"(v[0].x), "f"(v[0].y), "f"(v[1].x), "f"(v[1].y), "f"(v[2].x),
+                         "f"(v[2].y), "f"(v[3].x), "f"(v[3].y) : "memory");
+    } else if ((G & 1) == 0) {
+        if (g < G) *reinterpret_cast<float4 *>(row + g) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+        if (g + 2 < G)
+            *reinterpret_cast<float4 *>(row + g + 2) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
     } else {
-        if (g < G) row[g] = make_float2(v.x, v.y);
-        if (g + 1 < G) row[g + 1] = make_float2(v.z, v.w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (g + i < G) row[g + i] = v[i];
     }
 }
 
@@ -402,12 +413,14 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
                 tmem_ld16(lanebase + 3 * Gp + gb, im1);
                 if (valid) {
 #pragma unroll
-                    for (int i = 0; i < 16; i += 2)
-                        store_gathers(Yrow, gb + i, a.G,
-                                      make_float4(fmaf(w0, re0[i], w1 * re1[i]),
-                                                  fmaf(w0, im0[i], w1 * im1[i]),
-                                                  fmaf(w0, re0[i + 1], w1 * re1[i + 1]),
-                                                  fmaf(w0, im0[i + 1], w1 * im1[i + 1])));
+                    for (int i = 0; i < 16; i += 4) {
+                        float2 v[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            v[e] = make_float2(fmaf(w0, re0[i + e], w1 * re1[i + e]),
+                                               fmaf(w0, im0[i + e], w1 * im1[i + e]));
+                        store_gathers(Yrow, gb + i, a.G, a.wide, v);
+                    }
                 }
             }
             fence_before_sync();
@@ -611,10 +624,13 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
                     }
                     if (l < a.nq) {
 #pragma unroll
-                        for (int i = 0; i < 16; i += 2)
-                            store_gathers(Xrow, gb + i, a.G,
-                                          make_float4(a.scale * re[i], a.scale * im[i],
-                                                      a.scale * re[i + 1], a.scale * im[i + 1]));
+                        for (int i = 0; i < 16; i += 4) {
+                            float2 v[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                v[e] = make_float2(a.scale * re[i + e], a.scale * im[i + e]);
+                            store_gathers(Xrow, gb + i, a.G, a.wide, v);
+                        }
                     }
                 }
             }
@@ -648,6 +664,7 @@ static TcArgs tc_args(const Plan &p, bool adjoint, int *counter) {
     a.qn = p.qexplicit ? p.qn : nullptr;
     a.stall = p.tc_stall ? 1 : 0;
     a.wait_ns = p.tc_stall ? 20000000ull : 1000000000ull;   // 20 ms under the test hook, else 1 s
+    a.wide = 0;
     a.scale = (float)(1.0 / p.nfft);
     return a;
 }
@@ -676,7 +693,8 @@ cudaError_t configure_tc_kernels(Plan &p, int num_sms, int max_smem) {
 
 cudaError_t launch_slice_tc(Plan &p, bool adjoint, const float2 *in, float2 *out,
                             cudaStream_t st, int *counter) {
-    const TcArgs a = tc_args(p, adjoint, counter);
+    TcArgs a = tc_args(p, adjoint, counter);
+    a.wide = p.ngather % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 31) == 0;
     if (adjoint)
         slice_adj_tc_kernel<<<p.slice_grid_adj, kTcThreads, p.smem_sadj, st>>>(a, in, out);
     else
