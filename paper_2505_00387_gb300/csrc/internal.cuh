@@ -170,6 +170,9 @@ struct Plan {
     // groups above), and the blocked groups' number and log2(pairs)
     ColGroup *cg_model_pair = nullptr, *cg_data_pair = nullptr;
     int ncg_model_blk = 0, ncg_data_blk = 0, blk_lp = 0;
+    // tensor-core plans of short frames: pairs of neighbouring gathers
+    bool gather_frames = false;
+    int ncg_model_pair = 0, ncg_data_pair = 0;
     int frame_pairs = 0;           // column pairs per register-FFT block
     int frame_ahead = 0;           // such blocks resident on the device
     int frame_seq_model = 1, frame_seq_data = 1;   // pairs an analysis block takes in turn
@@ -276,6 +279,9 @@ cudaError_t configure_tile_kernels(Plan &p, int num_sms, int max_smem);
 // 1 synthesis, 2 both fused; bound: raise the plan's spectrum bound table
 bool frame_serves(int L, int nt, int ntau, int ns, int max_smem);
 cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem);
+// the same stages with the gathers fastest (tensor-core plans, row-major rows)
+bool gather_frames_serve(int L, int nt, int ntau, int ns, int max_smem);
+cudaError_t configure_gather_frames(Plan &p, int max_smem);
 cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *in, void *out,
                          const float *aux, const FistaArgs &fa, bool blocked, bool bound,
                          cudaStream_t st);

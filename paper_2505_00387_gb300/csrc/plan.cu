@@ -459,6 +459,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
     p->bins_fastest = !tc && (direct || (p->nos >= 32 && p->nos <= 512)) &&
                       frame_serves(p->L, p->nt, p->ntau, p->ns, optin);
+    p->gather_frames = tc && gather_frames_serve(p->L, p->nt, p->ntau, p->ns, optin);
     const size_t per_slice = (size_t)std::max(ld_interleaved(p->nos), ld_split(p->nos)) *
                              sizeof(float2);
     if (opts.theta_group > 0) {
@@ -557,7 +558,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
 
     // ------------------------------------------------- column groups
     const int cpg = 2 * p->pairs;
-    std::vector<ColGroup> cgm, cgd;
+    std::vector<ColGroup> cgm, cgd, cgmp, cgdp;
     if (tc) {
         // Real columns (q, theta, gather) and (trace, gather), gather fastest;
         // spectra slice-major, X[j][k][l][g] and Y[j][k][i][g] (i = the trace's
@@ -565,12 +566,6 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         // column group never straddles two (q, theta) or two traces.
         const int G = G_tc, J = p->ntheta, nq = p->nq;
         const long long nb = p->nbins;
-        for (int l = 0; l < nq; ++l)
-            for (int j = 0; j < J; ++j)
-                for (int g0 = 0; g0 < G; g0 += cpg)
-                    cgm.push_back(ColGroup{((long long)l * J + j) * G + g0,
-                                           ((long long)j * nb * nq + l) * G + g0, 0,
-                                           (int)(C * G), nq * G, std::min(cpg, G - g0), 0});
         const CubeGeo &cg0 = cg[0];
         std::vector<int> rank(p->ntr[0]), slice(p->ntr[0]);
         for (int j = 0; j < J; ++j)
@@ -578,14 +573,26 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
                 rank[cg0.sorted[t].col] = t - cg0.start[j];
                 slice[cg0.sorted[t].col] = j;
             }
-        for (int h = 0; h < p->ntr[0]; ++h) {
-            const int j = slice[h];
-            const int cnt = cg0.start[j + 1] - cg0.start[j];
-            for (int g0 = 0; g0 < G; g0 += cpg)
-                cgd.push_back(ColGroup{(long long)h * G + g0,
-                                       (nb * cg0.start[j] + rank[h]) * G + g0, 0,
-                                       p->ntr[0] * G, cnt * G, std::min(cpg, G - g0), 0});
-        }
+        auto gather_groups = [&](int cols, std::vector<ColGroup> *m, std::vector<ColGroup> *d) {
+            for (int l = 0; l < nq; ++l)
+                for (int j = 0; j < J; ++j)
+                    for (int g0 = 0; g0 < G; g0 += cols)
+                        m->push_back(ColGroup{((long long)l * J + j) * G + g0,
+                                              ((long long)j * nb * nq + l) * G + g0, 0,
+                                              (int)(C * G), nq * G, std::min(cols, G - g0), 0});
+            for (int h = 0; h < p->ntr[0]; ++h) {
+                const int j = slice[h];
+                const int cnt = cg0.start[j + 1] - cg0.start[j];
+                for (int g0 = 0; g0 < G; g0 += cols)
+                    d->push_back(ColGroup{(long long)h * G + g0,
+                                          (nb * cg0.start[j] + rank[h]) * G + g0, 0,
+                                          p->ntr[0] * G, cnt * G, std::min(cols, G - g0), 0});
+            }
+        };
+        gather_groups(cpg, &cgm, &cgd);
+        if (p->gather_frames) gather_groups(2, &cgmp, &cgdp);
+        p->ncg_model_pair = (int)cgmp.size();
+        p->ncg_data_pair = (int)cgdp.size();
     }
     auto column_groups = [&](int cols, std::vector<ColGroup> *m, std::vector<ColGroup> *d) {
         for (int c = 0; c < ncube; ++c)
@@ -619,7 +626,6 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     // the solver's blocked state: the same groups, or single pairs where the
     // register-FFT kernels run it
     const int bcols = p->bins_fastest ? 2 : cpg;
-    std::vector<ColGroup> cgmp, cgdp;
     if (p->bins_fastest) column_groups(2, &cgmp, &cgdp);
     std::vector<ColGroup> cgmb = p->bins_fastest ? cgmp : cgm, cgdb = p->bins_fastest ? cgdp : cgd;
     p->blk_lp = p->bins_fastest ? 0 : p->lp;
@@ -730,7 +736,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     }
     AAHRT_TRY(upload(&p->cg_model, cgm), "upload column groups");
     AAHRT_TRY(upload(&p->cg_data, cgd), "upload column groups");
-    if (p->bins_fastest) {
+    if (p->bins_fastest || p->gather_frames) {
         AAHRT_TRY(upload(&p->cg_model_pair, cgmp), "upload column groups");
         AAHRT_TRY(upload(&p->cg_data_pair, cgdp), "upload column groups");
         auto fractions = [](const std::vector<RowPos> &pos) {     // whole float4s
@@ -857,6 +863,8 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         p->tc_ntiles = (int)tiles.size();
         AAHRT_TRY(upload(&p->tc_tiles, tiles), "upload row tiles");
         AAHRT_TRY(configure_tc_kernels(*p, num_sms, max_smem), "tensor-core kernel configuration");
+        if (p->gather_frames)
+            AAHRT_TRY(configure_gather_frames(*p, max_smem), "time kernel configuration");
     } else if (direct) {
         AAHRT_TRY(configure_direct_kernels(*p, num_sms, max_smem), "direct kernel configuration");
         if (p->bins_fastest)

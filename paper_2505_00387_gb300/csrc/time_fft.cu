@@ -49,6 +49,22 @@ bool frame_serves(int L, int nt, int ntau, int ns, int max_smem) {
     return L >= 9 && L <= 13 && frame_plan_smem(L, 1, nt, ntau, ns) + 1024 <= (size_t)max_smem;
 }
 
+bool gather_frames_serve(int L, int nt, int ntau, int ns, int max_smem) {
+    return L >= 9 && L <= 11 && frame_plan_smem(L, 4096 >> L, nt, ntau, ns) + 1024 <= (size_t)max_smem;
+}
+
+cudaError_t configure_gather_frames(Plan &p, int max_smem) {
+    p.frame_pairs = 4096 >> p.L;
+    const FrameArgs none{};
+    cudaError_t e = cudaSuccess;
+    for (int op = GATHER_R2C; op <= GATHER_C2R; ++op)
+        for (int model = 0; model < 2; ++model)
+            for (int epi = 0; epi < 2 && !e; ++epi)
+                e = frame_pick(p.L)(FrameCall{(FrameOp)op, model != 0, p.interp, epi, 1, nullptr,
+                                              max_smem}, none, nullptr, nullptr, nullptr);
+    return e;
+}
+
 cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem) {
     // 256 threads a block, fewer while blocks are fewer than SMs
     const long long groups = std::min(p.ncg_model_blk, p.ncg_data_blk);
@@ -108,7 +124,14 @@ cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *
     a.tw = p.tw_t;
     a.fa = fa;
     // (the direct sum has no fixed point, so no bound to keep)
-    a.ybd = bound && p.slice_interp != AAHRT_SLICE_DIRECT ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
+    const bool keep = bound && p.slice_interp != AAHRT_SLICE_DIRECT;
+    a.ybd = keep ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
+    if (p.gather_frames) {
+        a.groups = model_side ? p.cg_model_pair : p.cg_data_pair;
+        a.ngroups = model_side ? p.ncg_model_pair : p.ncg_data_pair;
+        a.seq = 1;
+        op = op == FRAME_R2C ? GATHER_R2C : GATHER_C2R;
+    }
     return frame_pick(p.L)(FrameCall{(FrameOp)op, model_side, p.interp, epi, p.frame_pairs, st, 0}, a,
                            in, out, aux);
 }

@@ -55,11 +55,15 @@ struct FrameMem {
     float2 *stg;        // this pair's staged rows, row 0 at stg
 };
 // (seq > 1: the block takes that many pairs in turn and stages all their rows.)
-__host__ __device__ constexpr int staged_rows(int nrows) { return (nrows + 6) & ~1; }
+// (The strides put neighbouring pairs four banks apart modulo 16: LEN is 4
+// modulo 16, so rows are a multiple of 16 beside a frame, 4 more without one.)
+__host__ __device__ constexpr int staged_rows(int nrows) { return (nrows + 5 + 15) & ~15; }
+__host__ __device__ constexpr int turn_rows(int nrows) { return staged_rows(nrows) + 4; }
 template <class F>
 __host__ __device__ constexpr size_t frame_smem(int pairs, int seq, int nrows, int nfrac) {
     return (size_t)F::T * sizeof(float2) + (size_t)((nfrac + 3) & ~3) * sizeof(float) +
-           (size_t)pairs * (F::LEN + seq * staged_rows(nrows)) * sizeof(float2);
+           (size_t)pairs * (F::LEN + (seq > 1 ? seq * turn_rows(nrows) : staged_rows(nrows))) *
+               sizeof(float2);
 }
 template <class F>
 __device__ __forceinline__ FrameMem frame_mem(float4 *base, int pair, int nrows, int nfrac) {
@@ -310,15 +314,14 @@ __device__ __forceinline__ void frame_unstretch_t(const FrameMem &mem, const Dev
     __syncthreads();
 }
 
-// Analysis of the staged rows: resample onto the frame, FFT, unpack the two
-// real spectra to bins [0, nbins) of the pair's columns.
-template <class F, int INTERP, bool TRANS>
-__device__ __forceinline__ void frame_analyse(const FrameMem &mem, const ColGroup &cg, bool on,
-                                              const DevResampler &rs, const FrameScatter &sc,
-                                              int nrows, const float2 *__restrict__ tw, int nbins,
-                                              int t, float2 *__restrict__ out,
-                                              const FrameBound &ybd) {
-    constexpr int N = F::N, T = F::T;
+// Analysis of the staged rows up to the pair's spectrum Z (natural order, in
+// the frame): resample onto the frame, FFT; before_barrier() runs ahead of the
+// last barrier.
+template <class F, int INTERP, bool TRANS, class Fn>
+__device__ __forceinline__ void frame_spectrum(const FrameMem &mem, const DevResampler &rs,
+                                               const FrameScatter &sc, int nrows,
+                                               const float2 *__restrict__ tw, int t,
+                                               Fn before_barrier) {
     const FrameTwiddle ft = frame_twiddle<F>(tw, t);
     float2 v[16];
     if (TRANS) frame_unstretch_t<F, INTERP>(mem, rs, sc, nrows, t, v);
@@ -327,14 +330,37 @@ __device__ __forceinline__ void frame_analyse(const FrameMem &mem, const ColGrou
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; ++m) mem.sm[frame_at(frame_out<F>(m, t))] = v[m];
+    before_barrier();
+    __syncthreads();
+}
+
+// Bin k of the two real columns whose spectrum A + iB the frame holds:
+// A = (Z_k + conj Z_{N-k})/2, B = (Z_k - conj Z_{N-k})/(2i).
+template <class F>
+__device__ __forceinline__ float4 frame_bin(const float2 *sm, int k) {
+    const float2 zk = sm[frame_at(k)];
+    const float2 zn = sm[frame_at((F::N - k) & (F::N - 1))];
+    return make_float4(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y), 0.5f * (zk.y + zn.y),
+                       -0.5f * (zk.x - zn.x));
+}
+
+// Analysis of the staged rows: their spectrum, unpacked to bins [0, nbins) of
+// the pair's columns.
+template <class F, int INTERP, bool TRANS>
+__device__ __forceinline__ void frame_analyse(const FrameMem &mem, const ColGroup &cg, bool on,
+                                              const DevResampler &rs, const FrameScatter &sc,
+                                              int nrows, const float2 *__restrict__ tw, int nbins,
+                                              int t, float2 *__restrict__ out,
+                                              const FrameBound &ybd) {
+    constexpr int T = F::T;
     // (a block of several pairs has few chunks: pairs x chunks <= 128)
     __shared__ unsigned s_ymax[128];
     const bool bound = TRANS && ybd.max != nullptr;
     unsigned *ym = s_ymax + (threadIdx.x / T) * ybd.nchunk;
-    if (bound)
-        for (int i = t; i < ybd.nchunk; i += T) ym[i] = 0u;
-    __syncthreads();
-    // A = (Z_k + conj Z_{N-k})/2, B = (Z_k - conj Z_{N-k})/(2i)
+    frame_spectrum<F, INTERP, TRANS>(mem, rs, sc, nrows, tw, t, [&] {
+        if (bound)
+            for (int i = t; i < ybd.nchunk; i += T) ym[i] = 0u;
+    });
     const bool two = cg.ncol > 1;
     float2 *d0 = out + cg.bins_off, *d1 = d0 + nbins;
 #pragma unroll
@@ -342,10 +368,8 @@ __device__ __forceinline__ void frame_analyse(const FrameMem &mem, const ColGrou
         const int k = t + T * m;
         float amax = 0.f;
         if (on && k < nbins) {
-            const float2 zk = mem.sm[frame_at(k)];
-            const float2 zn = mem.sm[frame_at((N - k) & (N - 1))];
-            const float2 A = make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
-            const float2 B = make_float2(0.5f * (zk.y + zn.y), -0.5f * (zk.x - zn.x));
+            const float4 v = frame_bin<F>(mem.sm, k);
+            const float2 A = make_float2(v.x, v.y), B = make_float2(v.z, v.w);
             d0[k] = A;
             amax = fabsf(A.x) + fabsf(A.y);
             if (two) {
@@ -403,7 +427,8 @@ __device__ __forceinline__ void prefetch_l2(const void *p, long long bytes) {
 // (natural order, zero beyond the ns resampled samples and either side of
 // them).  Thread t's step-1 inputs are bins t + T a and, as
 // Z_{N-k} = conj A + i conj B, bins T a - t.
-template <class F>
+// INTER: the fetched bins of the two columns lie side by side (A at 2k, B at 2k + 1).
+template <class F, bool INTER = false>
 __device__ __forceinline__ void frame_synthesise(const FrameMem &mem, const ColGroup &cg,
                                                  const float2 *__restrict__ tw, int nbins, int ns,
                                                  int t) {
@@ -418,8 +443,8 @@ __device__ __forceinline__ void frame_synthesise(const FrameMem &mem, const ColG
         const int k = a < 8 ? t + T * a : N - t - T * a;       // 0 < k <= N/2 for a >= 8
         float2 A = make_float2(0.f, 0.f), B = A;
         if (k < nbins) {
-            A = mem.sm[k];
-            if (two) B = mem.sm[N / 2 + k];
+            A = mem.sm[INTER ? 2 * k : k];
+            if (two) B = mem.sm[INTER ? 2 * k + 1 : N / 2 + k];
         }
         if (a == 0 && t == 0) A.y = B.y = 0.f;
         v[a] = a < 8 ? make_float2(A.x - B.y, A.y + B.x) : make_float2(A.x + B.y, B.x - A.y);
@@ -541,7 +566,7 @@ frame_r2c_kernel(const FrameArgs a, const float *__restrict__ in, float2 *__rest
     extern __shared__ float4 smem_f4[];
     const int t = threadIdx.x % F::T, pair = threadIdx.x / F::T;
     FrameMem mem = frame_mem<F>(smem_f4, pair, a.nrows, a.nfrac);
-    const int rows = staged_rows(a.nrows);
+    const int rows = turn_rows(a.nrows);
     const int g0 = (blockIdx.x * (blockDim.x / F::T) + pair) * a.seq;
     const int lseq = a.seq == 4 ? 2 : a.seq == 2 ? 1 : 0;
     {
@@ -689,6 +714,116 @@ frame_fused_kernel(const FrameArgs a, float2 *spec, const float *__restrict__ au
     __syncthreads();
     frame_analyse<F, INTERP, !SYN_TRANS>(mem, b.cg, b.on, a.ana, a.sc, a.nrows, a.tw, a.nbins,
                                           b.t, spec, a.ybd);
+}
+
+// ---------------------------------------------------- gathers fastest
+// Plans whose spectra and rows hold the gathers fastest (the tensor-core
+// plans): a row, or a bin, of neighbouring pairs is contiguous.  A block owns
+// 256 / T neighbouring pairs; they are transformed each by its own T threads,
+// and moved by all threads with the pair fastest, so every access is a run of
+// the block's pairs.
+template <class F>
+struct GatherBlock {
+    static constexpr int PB = 256 / F::T;
+    int t, pair;             // this thread's transform
+    int io, row0;            // the pair it moves, and its first row or bin (steps of T)
+    bool on, io_on;
+    ColGroup cg, iog;
+    FrameMem mem, iom;
+    __device__ __forceinline__ GatherBlock(const FrameArgs &a, float4 *base, int nrows)
+        : t(threadIdx.x % F::T), pair(threadIdx.x / F::T), io(threadIdx.x % PB),
+          row0(threadIdx.x / PB) {
+        const int g = blockIdx.x * PB;
+        on = g + pair < a.ngroups;
+        io_on = g + io < a.ngroups;
+        cg = a.groups[on ? g + pair : 0];
+        iog = a.groups[io_on ? g + io : 0];
+        mem = frame_mem<F>(base, pair, nrows, a.nfrac);
+        iom = frame_mem<F>(base, io, nrows, a.nfrac);
+    }
+};
+
+template <class F, int INTERP, bool TRANS>
+__global__ void __launch_bounds__(256, 3)
+gather_r2c_kernel(const FrameArgs a, const float *__restrict__ in, float2 *__restrict__ out) {
+    extern __shared__ float4 smem_f4[];
+    const GatherBlock<F> b(a, smem_f4, a.nrows);
+    const ColGroup &cg = b.iog;
+    const bool two = cg.ncol > 1;
+    if (b.io_on) {
+        const float *src = in + cg.real_off;
+        const bool vec = two && ((cg.real_off | cg.ld_real) & 1) == 0;
+        for (int r = b.row0; r < a.nrows; r += F::T) {
+            const float *x = src + (long long)r * cg.ld_real;
+            float2 *dst = b.iom.stg + r;
+            if (vec) {
+                frame_cp<8>(dst, x);
+            } else {
+                frame_cp<4>(&dst->x, x);
+                if (two) frame_cp<4>(&dst->y, x + 1);
+                else dst->y = 0.f;
+            }
+        }
+    }
+    zero_pads(b.mem, a.nrows, b.t);
+    frame_tables<F>(b.mem.s_tw, a.tw);
+    if (TRANS) copy_fractions(b.mem.sfr, a.frac, a.nfrac);
+    frame_cp_wait();
+    __syncthreads();
+    frame_spectrum<F, INTERP, TRANS>(b.mem, a.ana, a.sc, a.nrows, a.tw, b.t, [] {});
+    if (!b.io_on) return;
+    float2 *dst = out + cg.spec_off;
+    const bool vec = two && ((cg.spec_off | cg.ld_spec) & 1) == 0;
+    for (int k = b.row0; k < a.nbins; k += F::T) {
+        const float4 v = frame_bin<F>(b.iom.sm, k);
+        float2 *d = dst + (long long)k * cg.ld_spec;
+        if (vec) {
+            *reinterpret_cast<float4 *>(d) = v;
+        } else {
+            d[0] = make_float2(v.x, v.y);
+            if (two) d[1] = make_float2(v.z, v.w);
+        }
+    }
+}
+
+template <class F, int INTERP, bool TRANS, int EPI>
+__global__ void __launch_bounds__(256, 4)
+gather_c2r_kernel(const FrameArgs a, const float2 *__restrict__ in, float *__restrict__ out,
+                  const float *__restrict__ aux) {
+    extern __shared__ float4 smem_f4[];
+    const GatherBlock<F> b(a, smem_f4, 0);
+    const ColGroup &cg = b.iog;
+    const bool two = cg.ncol > 1;
+    if (b.io_on) {
+        const float2 *src = in + cg.spec_off;
+        const bool vec = two && ((cg.spec_off | cg.ld_spec) & 1) == 0;
+        for (int k = b.row0; k < a.nbins; k += F::T) {
+            const float2 *x = src + (long long)k * cg.ld_spec;
+            float2 *dst = b.iom.sm + 2 * k;
+            if (vec) {
+                frame_cp<16>(dst, x);
+            } else {
+                frame_cp<8>(dst, x);
+                if (two) frame_cp<8>(dst + 1, x + 1);
+            }
+        }
+    }
+    frame_tables<F>(b.mem.s_tw, a.tw);
+    frame_synthesise<F, true>(b.mem, b.cg, a.tw, a.nbins, a.ns, b.t);
+    if (!b.io_on) return;
+    const bool vec = ((cg.real_off | cg.ld_real) & 1) == 0;
+    const int last = a.syn.nrows - 1;
+    int2 nxt = frame_entry<TRANS>(a.syn, min(b.row0, last));
+    for (int i = b.row0; i < a.syn.nrows; i += F::T) {
+        const long long o = cg.real_off + (long long)i * cg.ld_real;
+        const int2 e = nxt;
+        nxt = frame_entry<TRANS>(a.syn, min(i + F::T, last));
+        float2 x;
+        if (EPI == EPI_RESIDUAL) x = row_load(aux + o, two, vec);
+        float2 g = frame_row<INTERP, TRANS>(b.iom, a.frac, e);
+        if (EPI == EPI_RESIDUAL) g = make_float2(x.x - g.x, x.y - g.y);
+        row_store(out + o, g, two, vec);
+    }
 }
 
 }  // namespace aahrt

@@ -6,7 +6,8 @@
 
 namespace aahrt {
 
-enum FrameOp { FRAME_R2C, FRAME_C2R, FRAME_FUSED };
+// (GATHER_*: gathers fastest, frames of at most 2048 samples)
+enum FrameOp { FRAME_R2C, FRAME_C2R, FRAME_FUSED, GATHER_R2C, GATHER_C2R };
 
 struct FrameCall {
     FrameOp op;
@@ -19,7 +20,7 @@ struct FrameCall {
 template <class F, class K, class... A>
 cudaError_t frame_run(const FrameCall &c, const FrameArgs &a, int nrows, K *kern, A... args) {
     if (c.max_smem > 0) return raise_smem_limit(kern, c.max_smem);
-    const int per = c.pairs * a.seq;
+    const int per = c.pairs * a.seq;       // pairs a block owns
     const int grid = (a.ngroups + per - 1) / per;
     kern<<<grid, F::T * c.pairs, frame_smem<F>(c.pairs, a.seq, nrows, a.nfrac), c.st>>>(a, args...);
     return cudaGetLastError();
@@ -32,6 +33,22 @@ cudaError_t frame_interp(const FrameCall &c, const FrameArgs &a, const void *in,
     const float2 *ci = static_cast<const float2 *>(in);
     float *fo = static_cast<float *>(out);
     float2 *co = static_cast<float2 *>(out);
+    if (c.op >= GATHER_R2C) {
+        if constexpr (F::T <= 128) {
+            if (c.op == GATHER_R2C)
+                return c.model_side
+                           ? frame_run<F>(c, a, a.nrows, gather_r2c_kernel<F, INTERP, false>, fi, co)
+                           : frame_run<F>(c, a, a.nrows, gather_r2c_kernel<F, INTERP, true>, fi, co);
+            if (c.model_side)
+                return frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, true, EPI_STORE>, ci, fo, aux);
+            return c.epi == EPI_RESIDUAL
+                       ? frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, false, EPI_RESIDUAL>, ci,
+                                      fo, aux)
+                       : frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, false, EPI_STORE>, ci, fo,
+                                      aux);
+        }
+        return cudaErrorInvalidValue;
+    }
     if (c.op == FRAME_R2C)
         return c.model_side
                    ? frame_run<F>(c, a, a.nrows, frame_r2c_kernel<F, INTERP, false>, fi, co)

@@ -543,7 +543,7 @@ cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
         if (e) return e;
     }
     prof_begin(p, stage, st);
-    if (p.bins_fastest && !natural) {
+    if (p.gather_frames ? !blocked : p.bins_fastest && !natural) {
         const cudaError_t e = launch_frame(p, 0, model_side, EPI_STORE, in, out, nullptr,
                                            FistaArgs{}, blocked, !model_side, st);
         prof_end(p, st);
@@ -568,7 +568,7 @@ cudaError_t launch_c2r(Plan &p, bool model_side, const float2 *in, float *out,
     const size_t smem = model_side ? p.smem_c2r_model : p.smem_c2r_data;
     const int stage = model_side ? 5 : 2;
     prof_begin(p, stage, st);
-    if (p.bins_fastest && !natural) {
+    if (p.gather_frames ? !blocked : p.bins_fastest && !natural) {
         const cudaError_t e = launch_frame(p, 1, model_side, epi, in, out, aux, fa, blocked, false,
                                            st);
         prof_end(p, st);

@@ -62,3 +62,25 @@ def test_odd_bins():
     aligned only."""
     bins = {_run(500, 500, "keys", fmax=f).info.nbins % 2 for f in (20.0, 20.06)}
     assert bins == {0, 1}
+
+
+@pytest.mark.parametrize("nt,nfft", [(200, 512), (400, 1024), (800, 2048), (1600, 4096)])
+@pytest.mark.parametrize("ng,interp", [(5, "keys"), (6, "linear"), (8, "keys")])
+def test_gathers_fastest(nt, nfft, ng, interp):
+    """The same stages with the gathers fastest (512 to 2048 samples, and the
+    length beyond), for gathers in whole 32-byte sectors, whole 16-byte pairs
+    and neither: every gather of a tensor-core plan against the oracle (1e-4)."""
+    rng = np.random.default_rng(91)
+    hx, hy = syn.disc_offsets(rng, 9, 1500.0)
+    q0, dq = syn.q_axis(17)
+    g = syn.Gather(nt, 4.0 / nt, nt + 3, 17, q0, dq, 3, hx, hy)
+    p = oracle_plan(g, interp=interp)
+    gp = gpu_plan(g, interp=interp, ngather=ng, precision="split_bf16")
+    assert gp.info.nfft == nfft
+    m = rng.standard_normal((g.ntau, g.nq, g.ntheta, ng))
+    d = rng.standard_normal((nt, 9, ng))
+    df = host(gp.forward(dev(m)), d.shape)
+    ma = host(gp.adjoint(dev(d)), m.shape)
+    for i in (0, ng - 1):
+        assert rel(df[..., i], ops.forward(p, m[..., i])) < 1e-4
+        assert rel(ma[..., i], ops.adjoint(p, d[..., i])) < 1e-4
