@@ -220,13 +220,16 @@ int autotune_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
             if (make(o, &pc)) continue;          // candidate does not fit (shared memory)
             double ms = 0;
             rc = time_pair(*pc, m, d2, g, st, &ms);
+            // the register-FFT time kernels do not depend on time_pairs
+            const bool one_tp = pc->bins_fastest;
             free_plan(pc);
             if (rc) return rc;
             if (ms < best) {
                 best = ms;
                 best_tg = tg;
-                best_tp = tp;
+                best_tp = one_tp ? base.time_pairs : tp;
             }
+            if (one_tp) break;
         }
     if (best >= 1e300) return set_error(AAHRT_ERR_UNSUPPORTED, "autotuner: no candidate fits");
 
