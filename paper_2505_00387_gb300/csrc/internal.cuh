@@ -170,7 +170,7 @@ struct Plan {
     // groups above), and the blocked groups' number and log2(pairs)
     ColGroup *cg_model_pair = nullptr, *cg_data_pair = nullptr;
     int ncg_model_blk = 0, ncg_data_blk = 0, blk_lp = 0;
-    // tensor-core plans of short frames: pairs of neighbouring gathers
+    // tensor-core plans on the register-FFT kernels: pairs of neighbouring gathers
     bool gather_frames = false;
     int ncg_model_pair = 0, ncg_data_pair = 0;
     int frame_pairs = 0;           // column pairs per register-FFT block

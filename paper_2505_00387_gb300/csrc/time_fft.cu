@@ -49,12 +49,15 @@ bool frame_serves(int L, int nt, int ntau, int ns, int max_smem) {
     return L >= 9 && L <= 13 && frame_plan_smem(L, 1, nt, ntau, ns) + 1024 <= (size_t)max_smem;
 }
 
+static int gather_pairs(int L) { return L >= 12 ? 2 : 4096 >> L; }
+
 bool gather_frames_serve(int L, int nt, int ntau, int ns, int max_smem) {
-    return L >= 9 && L <= 11 && frame_plan_smem(L, 4096 >> L, nt, ntau, ns) + 1024 <= (size_t)max_smem;
+    return L >= 9 && L <= 13 &&
+           frame_plan_smem(L, gather_pairs(L), nt, ntau, ns) + 1024 <= (size_t)max_smem;
 }
 
 cudaError_t configure_gather_frames(Plan &p, int max_smem) {
-    p.frame_pairs = 4096 >> p.L;
+    p.frame_pairs = gather_pairs(p.L);
     const FrameArgs none{};
     cudaError_t e = cudaSuccess;
     for (int op = GATHER_R2C; op <= GATHER_C2R; ++op)

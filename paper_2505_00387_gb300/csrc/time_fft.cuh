@@ -719,12 +719,15 @@ frame_fused_kernel(const FrameArgs a, float2 *spec, const float *__restrict__ au
 // ---------------------------------------------------- gathers fastest
 // Plans whose spectra and rows hold the gathers fastest (the tensor-core
 // plans): a row, or a bin, of neighbouring pairs is contiguous.  A block owns
-// 256 / T neighbouring pairs; they are transformed each by its own T threads,
-// and moved by all threads with the pair fastest, so every access is a run of
-// the block's pairs.
+// 256 / T neighbouring pairs, at least two (a bin of two pairs is a whole
+// sector); they are transformed each by its own T threads, and moved by all
+// threads with the pair fastest, so every access is a run of the block's pairs.
 template <class F>
 struct GatherBlock {
-    static constexpr int PB = 256 / F::T;
+    static constexpr int PB = F::T >= 256 ? 2 : 256 / F::T;
+    static constexpr int THREADS = PB * F::T;
+    static constexpr int MINB = THREADS == 256 ? 4 : THREADS == 512 ? 2 : 1;
+    static constexpr int MINB_ANA = THREADS == 256 ? 3 : THREADS == 512 ? 2 : 1;
     int t, pair;             // this thread's transform
     int io, row0;            // the pair it moves, and its first row or bin (steps of T)
     bool on, io_on;
@@ -744,7 +747,7 @@ struct GatherBlock {
 };
 
 template <class F, int INTERP, bool TRANS>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(GatherBlock<F>::THREADS, GatherBlock<F>::MINB_ANA)
 gather_r2c_kernel(const FrameArgs a, const float *__restrict__ in, float2 *__restrict__ out) {
     extern __shared__ float4 smem_f4[];
     const GatherBlock<F> b(a, smem_f4, a.nrows);
@@ -787,7 +790,7 @@ gather_r2c_kernel(const FrameArgs a, const float *__restrict__ in, float2 *__res
 }
 
 template <class F, int INTERP, bool TRANS, int EPI>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(GatherBlock<F>::THREADS, GatherBlock<F>::MINB)
 gather_c2r_kernel(const FrameArgs a, const float2 *__restrict__ in, float *__restrict__ out,
                   const float *__restrict__ aux) {
     extern __shared__ float4 smem_f4[];

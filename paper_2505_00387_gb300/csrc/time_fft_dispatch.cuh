@@ -6,7 +6,7 @@
 
 namespace aahrt {
 
-// (GATHER_*: gathers fastest, frames of at most 2048 samples)
+// (GATHER_*: gathers fastest)
 enum FrameOp { FRAME_R2C, FRAME_C2R, FRAME_FUSED, GATHER_R2C, GATHER_C2R };
 
 struct FrameCall {
@@ -34,20 +34,17 @@ cudaError_t frame_interp(const FrameCall &c, const FrameArgs &a, const void *in,
     float *fo = static_cast<float *>(out);
     float2 *co = static_cast<float2 *>(out);
     if (c.op >= GATHER_R2C) {
-        if constexpr (F::T <= 128) {
-            if (c.op == GATHER_R2C)
-                return c.model_side
-                           ? frame_run<F>(c, a, a.nrows, gather_r2c_kernel<F, INTERP, false>, fi, co)
-                           : frame_run<F>(c, a, a.nrows, gather_r2c_kernel<F, INTERP, true>, fi, co);
-            if (c.model_side)
-                return frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, true, EPI_STORE>, ci, fo, aux);
-            return c.epi == EPI_RESIDUAL
-                       ? frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, false, EPI_RESIDUAL>, ci,
-                                      fo, aux)
-                       : frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, false, EPI_STORE>, ci, fo,
-                                      aux);
-        }
-        return cudaErrorInvalidValue;
+        if (c.op == GATHER_R2C)
+            return c.model_side
+                       ? frame_run<F>(c, a, a.nrows, gather_r2c_kernel<F, INTERP, false>, fi, co)
+                       : frame_run<F>(c, a, a.nrows, gather_r2c_kernel<F, INTERP, true>, fi, co);
+        if (c.model_side)
+            return frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, true, EPI_STORE>, ci, fo, aux);
+        return c.epi == EPI_RESIDUAL
+                   ? frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, false, EPI_RESIDUAL>, ci, fo,
+                                  aux)
+                   : frame_run<F>(c, a, 0, gather_c2r_kernel<F, INTERP, false, EPI_STORE>, ci, fo,
+                                  aux);
     }
     if (c.op == FRAME_R2C)
         return c.model_side

@@ -64,10 +64,11 @@ def test_odd_bins():
     assert bins == {0, 1}
 
 
-@pytest.mark.parametrize("nt,nfft", [(200, 512), (400, 1024), (800, 2048), (1600, 4096)])
+@pytest.mark.parametrize("nt,nfft", [(200, 512), (400, 1024), (800, 2048), (1600, 4096),
+                                     (3200, 8192), (6400, 16384)])
 @pytest.mark.parametrize("ng,interp", [(5, "keys"), (6, "linear"), (8, "keys")])
 def test_gathers_fastest(nt, nfft, ng, interp):
-    """The same stages with the gathers fastest (512 to 2048 samples, and the
+    """The same stages with the gathers fastest (512 to 8192 samples, and the
     length beyond), for gathers in whole 32-byte sectors, whole 16-byte pairs
     and neither: every gather of a tensor-core plan against the oracle (1e-4)."""
     rng = np.random.default_rng(91)
