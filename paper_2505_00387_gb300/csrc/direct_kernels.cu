@@ -39,12 +39,7 @@ struct DirectArgs {
     int *counter;
     long long total;
     int nbins, nq, ntheta, ngroup, tgroup, chunk;
-    int bins;                // spectra X[q][theta][bin], Y[trace][bin]
     float scale;
-    // offset of (column c, bin k) in a cube's spectrum of ncol columns
-    __device__ __forceinline__ long long at(long long c, int k, int ncol) const {
-        return bins ? c * nbins + k : (long long)k * ncol + c;
-    }
 };
 
 // (cos, sin) of 2 pi t 2^-32 for a signed fraction t of a cycle
@@ -84,19 +79,18 @@ direct_fwd_kernel(const DirectArgs a, const float2 *__restrict__ X, float2 *__re
         const int ncol = g.nj + extra;
         // stage X[k][l][ja + jj] (slice index mod ntheta) as Xs[jj][l], so a
         // trace walks its slices' curvatures at unit stride
-        const float2 *Xk = X + g.x_off;
-        const int ncx = a.nq * a.ntheta;
+        const float2 *Xk = X + g.x_off + (long long)k * a.nq * a.ntheta;
         for (int idx = threadIdx.x; idx < a.nq * ncol; idx += blockDim.x) {
             const int l = idx / ncol;
             const int jj = idx - l * ncol;
             int j = g.ja + jj;
             if (j >= a.ntheta) j -= a.ntheta;
-            Xs[jj * a.nq + l] = __ldg(Xk + a.at((long long)l * a.ntheta + j, k, ncx));
+            Xs[jj * a.nq + l] = __ldg(Xk + (long long)l * a.ntheta + j);
         }
         __syncthreads();
 
         const TraceGeo *geo = a.geo + g.geo_off;
-        float2 *Yk = Y + g.y_off;
+        float2 *Yk = Y + g.y_off + (long long)k * g.ntr;
         for (int t = g.f0 + threadIdx.x; t < g.f1; t += blockDim.x) {
             const TraceGeo tr = geo[t];
             const int jj0 = tr.j0 - g.ja;
@@ -134,7 +128,7 @@ direct_fwd_kernel(const DirectArgs a, const float2 *__restrict__ X, float2 *__re
             }
             const float sr = (ar[0] + ar[1]) + (ar[2] + ar[3]);
             const float si = (ai[0] + ai[1]) + (ai[2] + ai[3]);
-            Yk[a.at(tr.col, k, g.ntr)] = make_float2(a.scale * sr, a.scale * si);
+            Yk[tr.col] = make_float2(a.scale * sr, a.scale * si);
         }
         __syncthreads();
     }
@@ -162,7 +156,7 @@ direct_adj_kernel(const DirectArgs a, const float2 *__restrict__ Y, float2 *__re
         const int k = (int)(item - (long long)gi * a.nbins);
         const SliceGroup g = a.groups[gi];
         const TraceGeo *geo = a.geo + g.geo_off;
-        const float2 *Yk = Y + g.y_off;
+        const float2 *Yk = Y + g.y_off + (long long)k * g.ntr;
         const int *ss = a.slice_start + g.ss_off;
         const int nf = g.f1 - g.f0, ntot = nf + (g.e1 - g.e0);
         for (int idx = threadIdx.x; idx < a.nq * g.nj; idx += blockDim.x) {
@@ -181,7 +175,7 @@ direct_adj_kernel(const DirectArgs a, const float2 *__restrict__ Y, float2 *__re
                 const int p = c0 + i;
                 const int t = p < nf ? g.f0 + p : g.e0 + (p - nf);
                 const TraceGeo tr = geo[t];
-                const float2 y = __ldg(Yk + a.at(tr.col, k, g.ntr));
+                const float2 y = __ldg(Yk + tr.col);
                 s_y[i] = make_float4(a.scale * y.x, a.scale * y.y, tr.w0, tr.w1);
                 s_ph[i] = phase_consts((unsigned long long)k * tr.A, (unsigned long long)k * tr.B);
             }
@@ -237,13 +231,12 @@ direct_adj_kernel(const DirectArgs a, const float2 *__restrict__ Y, float2 *__re
             }
             __syncthreads();
         }
-        float2 *Xk = X + g.x_off;
+        float2 *Xk = X + g.x_off + (long long)k * a.nq * a.ntheta + g.ja;
         for (int idx = threadIdx.x; idx < a.nq * g.nj; idx += blockDim.x) {
             const int l = idx / g.nj;
             const int jj = idx - l * g.nj;
             const float2 u = acc0[idx], v = acc1[idx];
-            Xk[a.at((long long)l * a.ntheta + g.ja + jj, k, a.nq * a.ntheta)] =
-                make_float2(u.x + v.x, u.y + v.y);
+            Xk[(long long)l * a.ntheta + jj] = make_float2(u.x + v.x, u.y + v.y);
         }
         __syncthreads();
     }
@@ -283,7 +276,6 @@ cudaError_t launch_slice_direct(Plan &p, bool adjoint, const float2 *in, float2 
     a.ngroup = p.ngroup;
     a.tgroup = p.tgroup;
     a.chunk = p.direct_chunk;
-    a.bins = p.bins_fastest ? 1 : 0;
     a.scale = (float)(1.0 / p.nfft);
     if (adjoint)
         direct_adj_kernel<<<p.slice_grid_adj, kThreadsSlice, p.smem_sadj, st>>>(a, in, out);

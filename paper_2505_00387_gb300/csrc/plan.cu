@@ -457,7 +457,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     // --------------------------------------------------- azimuth groups
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
-    p->bins_fastest = !tc && (direct || (p->nos >= 32 && p->nos <= 512)) &&
+    p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512 &&
                       frame_serves(p->L, p->nt, p->ntau, p->ns, optin);
     p->gather_frames = tc && gather_frames_serve(p->L, p->nt, p->ntau, p->ns, optin);
     const size_t per_slice = (size_t)std::max(ld_interleaved(p->nos), ld_split(p->nos)) *
@@ -485,7 +485,7 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     }
     if (p->tgroup > kMaxGroupSlices) p->tgroup = kMaxGroupSlices;
     p->pull_group = p->tgroup;
-    if (p->bins_fastest && !direct) {
+    if (p->bins_fastest) {
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
         choose_tiles(*p, opts.theta_group > 0, ncube, sms);
@@ -865,8 +865,6 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
             AAHRT_TRY(configure_gather_frames(*p, max_smem), "time kernel configuration");
     } else if (direct) {
         AAHRT_TRY(configure_direct_kernels(*p, num_sms, max_smem), "direct kernel configuration");
-        if (p->bins_fastest)
-            AAHRT_TRY(configure_frame_kernels(*p, num_sms, max_smem), "time kernel configuration");
     } else if (p->bins_fastest) {
         AAHRT_TRY(configure_tile_kernels(*p, num_sms, max_smem), "slice kernel configuration");
         AAHRT_TRY(configure_frame_kernels(*p, num_sms, max_smem), "time kernel configuration");

@@ -426,7 +426,7 @@ cudaError_t launch_slice(Plan &p, bool adjoint, const float2 *in, float2 *out,
     const int stage = adjoint ? 4 : 1;
     int *ctr = counter ? counter : p.counters + slot;
     cudaError_t e = cudaSuccess;
-    if (p.bins_fastest && p.slice_interp != AAHRT_SLICE_DIRECT) {
+    if (p.bins_fastest) {
         // the plan's own counter is left cleared by every launch
         if (counter && (e = cudaMemsetAsync(ctr, 0, (kDoneSlot + 1) * sizeof(int), st))) return e;
         prof_begin(p, stage, st);

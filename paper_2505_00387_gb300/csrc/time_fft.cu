@@ -126,9 +126,7 @@ cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *
     a.nbins = p.nbins;
     a.tw = p.tw_t;
     a.fa = fa;
-    // (the direct sum has no fixed point, so no bound to keep)
-    const bool keep = bound && p.slice_interp != AAHRT_SLICE_DIRECT;
-    a.ybd = keep ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
+    a.ybd = bound ? FrameBound{p.ymax, p.nychunk, p.ychunk_log} : FrameBound{nullptr, 0, 0};
     if (p.gather_frames) {
         a.groups = model_side ? p.cg_model_pair : p.cg_data_pair;
         a.ngroups = model_side ? p.ncg_model_pair : p.ncg_data_pair;
