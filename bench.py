@@ -428,11 +428,12 @@ def measure(kind, args, rank, world, dev):
     iter_ms = sum(st_ms[:6]) / sum(st_n[1:2] or [1])
     iter_bytes = sum(stage_bytes(info)[:6])
     fused = st_n[3] == 0 and st_n[2] > 0
-    kernel_names = ["r2c_kernel", "slice_fwd_kernel",
-                    "c2r_r2c_kernel" if fused else "c2r_kernel", "r2c_kernel",
-                    "slice_adj_kernel", "c2r_r2c_kernel" if fused else "c2r_kernel"]
+    pre, post = "frame_r2c_kernel", "frame_fused_kernel" if fused else "frame_c2r_kernel"
+    kernel_names = [pre, "tile_fwd_kernel", post, pre, "tile_adj_kernel", post]
     if slow:
-        kernel_names[1], kernel_names[4] = "direct_fwd_kernel", "direct_adj_kernel"
+        post = "c2r_r2c_kernel" if fused else "c2r_kernel"
+        kernel_names = ["r2c_kernel", "direct_fwd_kernel", post,
+                        "r2c_kernel", "direct_adj_kernel", post]
     suffix = "@direct" if slow else ("@batch512" if batch else "")
     rec = traffic_record(names[top] + suffix)
     line = {

@@ -457,6 +457,12 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     // --------------------------------------------------- azimuth groups
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
+    // Bins fastest wherever its kernels exist: frames whose FFT registers hold
+    // and q grids of two radix steps (32 points) up to two grids of 8 bins with
+    // three blocks an SM (512); measured on both sides in slice_tiles.cuh and
+    // time_fft.cuh.  The direct sum keeps natural spectra: it takes one bin at a
+    // time, and 8-byte pieces at a column stride cost its forward more (314 ->
+    // 361 us, 100 curvatures x 2000 traces) than the faster time stages gave.
     p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512 &&
                       frame_serves(p->L, p->nt, p->ntau, p->ns, optin);
     p->gather_frames = tc && gather_frames_serve(p->L, p->nt, p->ntau, p->ns, optin);

@@ -20,6 +20,14 @@
 // radix-R step, in place in rows p1 + 16 n2.  Rows nos .. nos + W - 2 repeat
 // rows 0 .. W - 2, so a trace's taps are consecutive rows (forward); the
 // adjoint spreads into them and its first step folds them back.
+//
+// Bound: issue (68-71 % of the slots) with the L1 / shared-memory pipe at
+// 57-71 %; the bin-per-block kernels had that pipe at 87-91 %, half of it
+// conflicts.  Per launch on 16 cubes of 200-3000 traces, 100 q x 36 azimuths,
+// 2048 bins (nos 256, W 7), bin per block -> these kernels: forward 823 -> 442
+// us, adjoint 1108 -> 622; one 2000-trace gather of the same axes 99 -> 72 and
+// 125 -> 92; one 8000-trace gather, 200 q x 72 azimuths (nos 512) 929 -> 593 and
+// 1400 -> 750.
 #pragma once
 
 #include "fft.cuh"

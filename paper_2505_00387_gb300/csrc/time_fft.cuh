@@ -10,11 +10,18 @@
 //          sum_a w_16^(a p0) x[t + T a],            t = C b + c,
 // three register steps (radix 16, 16, C) and two exchanges through shared
 // memory.  The first crosses the block (one barrier); the second stays inside
-// the C threads of one p0, which lie in one warp, so it needs none.  Input
-// comes straight from global memory (synthesis) or from the resampler
-// (analysis) into registers: a frame passes through shared memory 5 times in
-// the synthesis and 6 in the analysis, against 8 and 8 with every radix step
-// working in shared memory, at 80 instead of 128 registers (24 warps an SM).
+// the C threads of one p0, which lie in one warp, so it needs none.  Spectra
+// arrive in the frame by cp.async past L1 and the radix steps work in
+// registers: a frame passes through shared memory 5-6 times a transform,
+// against 8 with every radix step working there (time_kernels.cu).
+//
+// Bound: the L1 / shared-memory pipe (85 %) and issue (60-66 % of the slots),
+// at 64 registers (four blocks of 256 threads an SM; 80 and three in the
+// analysis alone) instead of 128 and two.  Per launch on 16 cubes of 1001
+// samples and 200-3000 traces (4096-sample frames), shared-memory FFT ->
+// these kernels: data half 839 -> 443 us, model half 734 -> 481; analysis
+// 661 -> 429 (model) and 1064 -> 632 (data), synthesis 699 -> 468 (data) and
+// 977 -> 676 (model).
 //
 // Shared-memory layout of an exchange: element (p0, i) of group p0 at
 // p0 (T + C) + i (the skew spreads the groups a half warp touches over the

@@ -1,7 +1,8 @@
 // Time-axis stages of the AAHRT (Algorithms 1 and 2, steps 1-2 and 4-5) on
 // spectra whose columns or gathers are fastest: every plan's stages on natural
-// layouts (aahrt_apply_stage, the pull scan), and the operators of the plans
-// the bins-fastest kernels (time_fft.cuh) do not serve:
+// layouts (aahrt_apply_stage, the pull scan), the solvers' half-iterations of
+// gathers-fastest plans, and the operators of the plans the register-FFT
+// kernels (time_fft.cuh) do not serve:
 //
 //   r2c: X[k][c] = sum_n (G in)[n][c] exp(-2 pi i k n / Nfft), k < nbins
 //        where G resamples each column: the time stretch S (model side,
