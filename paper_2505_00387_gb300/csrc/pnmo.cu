@@ -29,12 +29,19 @@ struct PnArgs {
 };
 
 constexpr int kPnRows = 8;            // rows a thread takes of its column
+constexpr int kPnCols = 8;            // columns of a block of the transpose
 
-// One thread owns kPnRows neighbouring rows of a column, so the column's
-// coefficient q_ref r^2/dt^2, as (hi, lo), is formed once and no index is
-// divided (a flat index cost a 64-bit division a sample, and the coefficients
-// a launch of their own: 34 us a call of a 2000-trace, 1001-sample gather, 25
-// now).
+// Forward: one thread owns kPnRows neighbouring rows of a column, so the
+// column's coefficient q_ref r^2/dt^2, as (hi, lo), is formed once and no index
+// is divided (a flat index cost a 64-bit division a sample, and the
+// coefficients a launch of their own: 29 us a call of a 2000-trace, 1001-sample
+// gather, 21 now).  The transpose evaluates five or six positions a sample, so
+// the coefficient is a small part and the serial chain is what counts: one row
+// a thread, in blocks of kPnCols columns x 16 rows.  Per call, flat index /
+// eight rows a thread / 32 columns / 16 / 8: 256 traces x 256 samples 23 / 100 /
+// 19 / 20 / 19 us, the gather 103 / 183 / 89 / 85 / 80, 16 cubes of 200-3000
+// traces 1002 / 1054 / 1014 / 958 / 906, 256 cubes of 33 traces x 100 samples
+// 33 / 62 / 39 / 35 / 33, 8000 traces x 2048 samples 928 / 764 / 764 / 694 / 633.
 __device__ __forceinline__ float2 pn_coef(const PnArgs &a, const PnBlock &b, int col) {
     const double v = a.q_ref * __ldg(a.rho + b.r0 + col / b.rep);
     const float hi = (float)v;
@@ -112,31 +119,29 @@ __global__ void __launch_bounds__(128)
 pnmo_t_kernel(const PnArgs a, const float *__restrict__ in, float *__restrict__ out) {
     constexpr int T0 = Taps<INTERP>::t0, TN = Taps<INTERP>::n;
     const PnBlock b = a.blk[blockIdx.z];
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= b.ld) return;
+    const int col = blockIdx.x * kPnCols + threadIdx.x % kPnCols;
+    const int r = blockIdx.y * (128 / kPnCols) + threadIdx.x / kPnCols;   // sample receiving
+    if (col >= b.ld || r >= a.nt) return;
     const float2 c = pn_coef(a, b, col);
-    const int r1 = min(a.nt, kPnRows * (int)(blockIdx.y + 1));
-    for (int r = kPnRows * blockIdx.y; r < r1; ++r) {        // input sample receiving
-        const float cc = c.x + c.y;
-        // outputs i read sample r when base_i + t = r for a tap t, i.e.
-        // u_i in [r - T0 - TN + 1, r - T0 + 1); one sample of margin each side
-        const float ulo = fmaxf((float)(r - T0 - TN), 0.f);
-        const float uhi = (float)(r - T0 + 2);
-        int ilo = isqrt_floor(ulo * ulo - cc) - 1;
-        int ihi = isqrt_floor(uhi * uhi - cc) + 1;
-        if (ilo < 0) ilo = 0;
-        if (ihi > a.nt - 1) ihi = a.nt - 1;
-        float v = 0.f;
-        for (int i = ilo; i <= ihi; ++i) {
-            int base;
-            float fr;
-            if (!pn_position(i, c, &base, &fr)) continue;
-            const int t = r - base;
-            if (t < T0 || t >= T0 + TN) continue;
-            v = fmaf(tap_weight<INTERP>(t, fr), __ldg(in + b.off + (long long)i * b.ld + col), v);
-        }
-        out[b.off + (long long)r * b.ld + col] = v;
+    const float cc = c.x + c.y;
+    // outputs i read sample r when base_i + t = r for a tap t, i.e.
+    // u_i in [r - T0 - TN + 1, r - T0 + 1); one sample of margin each side
+    const float ulo = fmaxf((float)(r - T0 - TN), 0.f);
+    const float uhi = (float)(r - T0 + 2);
+    int ilo = isqrt_floor(ulo * ulo - cc) - 1;
+    int ihi = isqrt_floor(uhi * uhi - cc) + 1;
+    if (ilo < 0) ilo = 0;
+    if (ihi > a.nt - 1) ihi = a.nt - 1;
+    float v = 0.f;
+    for (int i = ilo; i <= ihi; ++i) {
+        int base;
+        float fr;
+        if (!pn_position(i, c, &base, &fr)) continue;
+        const int t = r - base;
+        if (t < T0 || t >= T0 + TN) continue;
+        v = fmaf(tap_weight<INTERP>(t, fr), __ldg(in + b.off + (long long)i * b.ld + col), v);
     }
+    out[b.off + (long long)r * b.ld + col] = v;
 }
 
 }  // namespace aahrt
@@ -187,9 +192,10 @@ extern "C" int aahrt_partial_nmo(aahrt_plan *plan, const float *in, float *out, 
     cudaStream_t st = (cudaStream_t)stream;
     const PnArgs a{p.pn_blk, p.pn_rho, q_ref, p.nt};
     // (eight rows a thread pay for its coefficient and still give 2000 blocks
-    // from one 2000-trace gather)
-    const dim3 grid((unsigned)((p.pn_ldmax + 127) / 128),
-                    (unsigned)((p.nt + kPnRows - 1) / kPnRows), (unsigned)p.pn_nblk);
+    // from one 2000-trace gather; the transpose takes one row a thread)
+    const int cols = transpose ? kPnCols : 128, rows = transpose ? 128 / kPnCols : kPnRows;
+    const dim3 grid((unsigned)((p.pn_ldmax + cols - 1) / cols),
+                    (unsigned)((p.nt + rows - 1) / rows), (unsigned)p.pn_nblk);
     const bool keys = p.interp == AAHRT_INTERP_KEYS;
     if (transpose) {
         if (keys) pnmo_t_kernel<AAHRT_INTERP_KEYS><<<grid, 128, 0, st>>>(a, in, out);
