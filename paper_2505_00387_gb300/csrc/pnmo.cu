@@ -49,7 +49,9 @@ __device__ __forceinline__ float2 pn_coef(const PnArgs &a, const PnBlock &b, int
 }
 
 // Position u = sqrt(i^2 + c) of output row i as base + frac, frac in [0, 1);
-// false where i^2 + c < 0 (the output is muted).
+// false where i^2 + c < 0 (the output is muted), or where u is beyond every
+// record (nt < 46341) or not a number (c past the float range), so that base
+// stays far from the ends of the integers.
 __device__ __forceinline__ bool pn_position(int i, float2 c, int *base, float *frac) {
     const int ii = i * i;
     const float a_hi = __int2float_rn(ii);
@@ -58,7 +60,8 @@ __device__ __forceinline__ bool pn_position(int i, float2 c, int *base, float *f
     const float bb = __fsub_rn(s, a_hi);
     const float err = __fadd_rn(__fsub_rn(a_hi, __fsub_rn(s, bb)), __fsub_rn(c.x, bb));
     const float t = __fadd_rn(__fadd_rn(err, a_lo), c.y);
-    if (__fadd_rn(s, t) < 0.f) return false;
+    const float u2 = __fadd_rn(s, t);
+    if (!(u2 >= 0.f && u2 < 4294967296.f)) return false;
     const float u0 = sqrtf(fmaxf(s, 0.f));
     float corr = 0.f;
     if (u0 > 0.f) corr = __fadd_rn(__fmaf_rn(-u0, u0, s), t) / __fmul_rn(2.f, u0);
@@ -105,9 +108,11 @@ pnmo_kernel(const PnArgs a, const float *__restrict__ in, float *__restrict__ ou
 }
 
 // largest i >= 0 with i^2 <= x (x may be negative: -1), by a float root and
-// integer corrections
+// integer corrections; beyond 46341^2 (nt is below 46341) some i > nt, since a
+// root past the 32-bit range would leave the corrections without an end
 __device__ __forceinline__ int isqrt_floor(float x) {
     if (x < 0.f) return -1;
+    x = fminf(x, 2147580964.f);          // 46342^2
     int r = (int)sqrtf(x);
     while ((float)r * r > x) --r;
     while ((float)(r + 1) * (r + 1) <= x) ++r;
