@@ -452,6 +452,12 @@ int aahrt_plan_status(aahrt_plan *plan);
  * production use. */
 int aahrt_plan_test_stall(aahrt_plan *plan, int on);
 
+/* Test hook for a failed kernel launch: while on, the plan's slice adjoints
+ * are not launched and the calls that need one return AAHRT_ERR_CUDA, with the
+ * kernels before it already queued (a solve already captured in the plan's
+ * graph is not affected).  Not for production use. */
+int aahrt_plan_test_fail_adjoint(aahrt_plan *plan, int on);
+
 const char *aahrt_status_string(int status);
 const char *aahrt_last_error(void);
 

@@ -888,6 +888,13 @@ int aahrt_plan_test_stall(aahrt_plan *plan, int on) {
     return AAHRT_OK;
 }
 
+int aahrt_plan_test_fail_adjoint(aahrt_plan *plan, int on) {
+    if (!plan) return set_error(AAHRT_ERR_INVALID_ARG, "plan is NULL");
+    if (on != 0 && on != 1) return set_error(AAHRT_ERR_INVALID_ARG, "on must be 0 or 1");
+    plan->p->fail_adj = on != 0;
+    return AAHRT_OK;
+}
+
 const char *aahrt_status_string(int status) {
     switch (status) {
         case AAHRT_OK: return "success";

@@ -157,6 +157,10 @@ struct Plan {
     unsigned *ymax = nullptr;
     float *wsum = nullptr;
     int nychunk = 0, ychunk_log = 6;
+    // Bins-fastest plans: the slice adjoint that reads the table clears it.
+    // raised: an analysis wrote the table and no slice adjoint has been
+    // launched since; stale: it may hold values no slice adjoint has cleared.
+    bool ybound_raised = false, ybound_stale = false;
     int ngroups_total = 0;
     long long slice_items = 0;
     int *counters = nullptr;       // work counters of the persistent kernels
@@ -220,6 +224,7 @@ struct Plan {
     double *pn_rho = nullptr;      // [traces of every distinct geometry]
     int tc_gp = 0;                 // gathers padded to a multiple of 8
     int4 *tc_tiles = nullptr;      // forward row tiles {slice, first, end, 0}
+    bool fail_adj = false;         // test hook: slice adjoints report a failed launch
     bool tc_stall = false;         // test hook: tensor-core kernels issue no MMAs
     int tc_ntiles = 0;
     // deconvolutive operator: wavelet convolved with every trace in time
@@ -336,6 +341,13 @@ int noalloc_prepare(int dev);
 // Spectrum bound table of the slice adjoint computed from a given Y (when Y
 // does not come from the data-side analysis, which writes the table itself).
 cudaError_t launch_ybound(Plan &p, const float2 *Y, cudaStream_t st);
+
+// Before a kernel of a bins-fastest plan raises the bound table.  The slice
+// adjoint that reads the table leaves it cleared, so no memset stands between
+// the kernels; but when that adjoint was never launched (a launch in between
+// failed), the old values are still there and the next adjoint would lose bits
+// to a bound that is too large: then the table is cleared here.
+cudaError_t ybound_begin(Plan &p, cudaStream_t st);
 
 // operator application used by the C ABI and the solver
 int apply_forward(Plan &p, const float *m, float *d, cudaStream_t st,

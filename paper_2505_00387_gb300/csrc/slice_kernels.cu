@@ -382,9 +382,27 @@ __global__ void ybound_kernel(const SliceGroup *__restrict__ groups,
         atomicMax(ymax + (long long)g.cube * nchunk + blockIdx.y, __float_as_uint(m));
 }
 
+cudaError_t ybound_begin(Plan &p, cudaStream_t st) {
+    p.ybound_stale |= p.ybound_raised;
+    if (p.ybound_stale) {
+        const cudaError_t e =
+            cudaMemsetAsync(p.ymax, 0, (size_t)p.ncube * p.nychunk * sizeof(unsigned), st);
+        if (e) return e;
+        // (a captured memset clears the table when the graph runs, not now)
+        cudaStreamCaptureStatus cap;
+        if (!cudaStreamIsCapturing(st, &cap) && cap == cudaStreamCaptureStatusNone)
+            p.ybound_stale = false;
+    }
+    p.ybound_raised = true;
+    return cudaSuccess;
+}
+
 cudaError_t launch_ybound(Plan &p, const float2 *Y, cudaStream_t st) {
     if (!p.ymax || p.precision == 1 || p.slice_interp == AAHRT_SLICE_DIRECT) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(p.ymax, 0, (size_t)p.ncube * p.nychunk * sizeof(unsigned), st);
+    cudaError_t e = p.bins_fastest
+                        ? ybound_begin(p, st)
+                        : cudaMemsetAsync(p.ymax, 0,
+                                          (size_t)p.ncube * p.nychunk * sizeof(unsigned), st);
     if (e) return e;
     ybound_kernel<<<dim3(p.ngroups_total, p.nychunk), 256, 0, st>>>(
         p.groups, Y, p.nbins, p.ychunk_log, p.nychunk, p.ymax);
@@ -426,11 +444,13 @@ cudaError_t launch_slice(Plan &p, bool adjoint, const float2 *in, float2 *out,
     const int stage = adjoint ? 4 : 1;
     int *ctr = counter ? counter : p.counters + slot;
     cudaError_t e = cudaSuccess;
+    if (adjoint && p.fail_adj) return cudaErrorLaunchOutOfResources;
     if (p.bins_fastest) {
         // the plan's own counter is left cleared by every launch
         if (counter && (e = cudaMemsetAsync(ctr, 0, (kDoneSlot + 1) * sizeof(int), st))) return e;
         prof_begin(p, stage, st);
         e = launch_slice_tiles(p, adjoint, in, out, st, ctr);
+        if (adjoint && !e) p.ybound_raised = false;
         prof_end(p, st);
         p.launches[stage]++;
         return e;

@@ -537,10 +537,10 @@ cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
     const size_t smem = model_side ? p.smem_r2c_model : p.smem_r2c_data;
     const int stage = model_side ? 0 : 3;
     YBound yb{};
-    // (bins-fastest plans: the slice adjoint leaves the table cleared, and
-    // aahrt_apply_stage computes it from the spectrum it is given)
-    if (!model_side && !p.bins_fastest) {
-        const cudaError_t e = ybound_reset(p, st, &yb);
+    // (natural spectra of bins-fastest plans: aahrt_apply_stage computes the
+    // bound from the spectrum it is given)
+    if (!model_side && !(p.bins_fastest && natural)) {
+        const cudaError_t e = p.bins_fastest ? ybound_begin(p, st) : ybound_reset(p, st, &yb);
         if (e) return e;
     }
     prof_begin(p, stage, st);
@@ -619,8 +619,8 @@ cudaError_t launch_c2r_r2c(Plan &p, bool model_side, float2 *spec, const float *
     const int n = model_side ? p.ncg_model : p.ncg_data;
     const int stage = model_side ? 5 : 2;
     YBound yb{};
-    if (!model_side && !p.bins_fastest) {
-        const cudaError_t e = ybound_reset(p, st, &yb);
+    if (!model_side) {
+        const cudaError_t e = p.bins_fastest ? ybound_begin(p, st) : ybound_reset(p, st, &yb);
         if (e) return e;
     }
     prof_begin(p, stage, st);
