@@ -44,6 +44,16 @@ __host__ __device__ __forceinline__ int ld_split(int n) {
 }
 
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+    return make_float2(a.x + b.x, a.y + b.y);
+}
+__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
+    return make_float2(a.x - b.x, a.y - b.y);
+}
+// The same sums as one two-wide instruction (3-5 % of a register-FFT kernel).
+// Each half rounds like the scalar add, but no product before it can be
+// contracted into it: a network of these rounds its multiplications by
+// sqrt(1/2) once more, so the block FFTs below keep the scalar forms.
+__host__ __device__ __forceinline__ float2 cadd2(float2 a, float2 b) {
 #ifdef __CUDA_ARCH__
     float2 r;
     asm("{.reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; add.rn.f32x2 z, x, y; "
@@ -51,10 +61,10 @@ __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) {
         : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return r;
 #else
-    return make_float2(a.x + b.x, a.y + b.y);
+    return cadd(a, b);
 #endif
 }
-__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
+__host__ __device__ __forceinline__ float2 csub2(float2 a, float2 b) {
 #ifdef __CUDA_ARCH__
     float2 r;
     asm("{.reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; sub.rn.f32x2 z, x, y; "
@@ -62,7 +72,7 @@ __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
         : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return r;
 #else
-    return make_float2(a.x - b.x, a.y - b.y);
+    return csub(a, b);
 #endif
 }
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
@@ -185,8 +195,8 @@ __host__ __device__ __forceinline__ int rev_bits_c(int m) {
     return r;
 }
 
-// Constant radix-2^A DIF network on v[0..2^A) (in place).
-template <int A, bool INV>
+// Constant radix-2^A DIF network on v[0..2^A) (in place); PACK: two-wide adds.
+template <int A, bool INV, bool PACK = false>
 __host__ __device__ __forceinline__ void dif_network(float2 *v) {
     constexpr int R = 1 << A;
 #pragma unroll
@@ -197,8 +207,8 @@ __host__ __device__ __forceinline__ void dif_network(float2 *v) {
         for (int m = 0; m < R; ++m) {
             if (m & Mt) continue;
             const float2 a = v[m], c = v[m + Mt];
-            v[m] = cadd(a, c);
-            v[m + Mt] = kappa_mul<INV>(csub(a, c), T, m & (Mt - 1));
+            v[m] = PACK ? cadd2(a, c) : cadd(a, c);
+            v[m + Mt] = kappa_mul<INV>(PACK ? csub2(a, c) : csub(a, c), T, m & (Mt - 1));
         }
     }
 }

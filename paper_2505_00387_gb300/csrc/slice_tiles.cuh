@@ -114,8 +114,8 @@ __device__ __forceinline__ void dif16_centred(float2 *v) {
         v[m] = v[m + 8];
         v[m + 8] = kappa_mul<INV>(make_float2(-v[m].x, -v[m].y), 3, m);
     }
-    dif_network<3, INV>(v);
-    dif_network<3, INV>(v + 8);
+    dif_network<3, INV, true>(v);
+    dif_network<3, INV, true>(v + 8);
 }
 
 // Half of a radix-32 DFT (nos = 512): v[n] = (x[n] +- x[n + 16]) w_32^(n b),
@@ -126,10 +126,10 @@ __device__ __forceinline__ void half_of_32(float2 *v, int b, const float2 *s_tw,
     for (int n = 0; n < 16; ++n) {
         const float2 p = x(n), q = x(n + 16);
         if (b == 0) {
-            v[n] = cadd(p, q);
+            v[n] = cadd2(p, q);
         } else {
             const float2 w = s_tw[16 * 16 + n];
-            v[n] = cmul(csub(p, q), make_float2(w.x, INV ? -w.y : w.y));
+            v[n] = cmul(csub2(p, q), make_float2(w.x, INV ? -w.y : w.y));
         }
     }
 }
@@ -147,7 +147,7 @@ __device__ __forceinline__ void tile_fwd_step2(float2 *G, const float2 *s_tw, in
         float2 *col = G + p1 * TB + bin;
         float2 v[16];
         half_of_32<false>(v, b, s_tw, [&](int n) { return col[n * 16 * TB]; });
-        dif_network<4, false>(v);
+        dif_network<4, false, true>(v);
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < 16; ++m) col[(2 * rev_bits_c<4>(m) + b) * 16 * TB] = v[m];
@@ -161,7 +161,7 @@ __device__ __forceinline__ void tile_fwd_step2(float2 *G, const float2 *s_tw, in
             float2 v[R];
 #pragma unroll
             for (int n = 0; n < R; ++n) v[n] = col[n * 16 * TB];
-            dif_network<T::LR, false>(v);
+            dif_network<T::LR, false, true>(v);
 #pragma unroll
             for (int m = 0; m < R; ++m) col[rev_bits_c<T::LR>(m) * 16 * TB] = v[m];
             if (p1 < T::W - 1) col[T::NOS * TB] = v[0];
@@ -200,7 +200,7 @@ __device__ __forceinline__ void tile_fwd_grid(const TileArgs &a, const float2 *_
             v[m].y *= d;
         }
         if (centred) dif16_centred<false>(v);
-        else dif_network<4, false>(v);
+        else dif_network<4, false, true>(v);
         float2 *col = G + (n2 << 4) * TB + bin;
         const float2 *tw = s_tw + (n2 << 4);
 #pragma unroll
@@ -349,7 +349,7 @@ __device__ __forceinline__ void tile_adj_step1(float2 *G, int sub, int bin, cons
         const PlanePair<TB> pl(reinterpret_cast<const int *>(G + p1 * TB) + bin);
         float2 v[16];
         half_of_32<true>(v, b, s_tw, [&](int n) { return fixed(pl, p1, n); });
-        dif_network<4, true>(v);
+        dif_network<4, true, true>(v);
         __syncthreads();
         float2 *col = G + p1 * TB + bin;
         if (b == 0 && p1 < T::W - 1) col[T::NOS * TB] = make_float2(0.f, 0.f);
@@ -367,7 +367,7 @@ __device__ __forceinline__ void tile_adj_step1(float2 *G, int sub, int bin, cons
             float2 v[R];
 #pragma unroll
             for (int n = 0; n < R; ++n) v[n] = fixed(pl, p1, n);
-            dif_network<T::LR, true>(v);
+            dif_network<T::LR, true, true>(v);
             float2 *col = G + p1 * TB + bin;
             __syncwarp();        // the row's lanes have read it
             if (p1 < T::W - 1) col[T::NOS * TB] = make_float2(0.f, 0.f);
@@ -397,7 +397,7 @@ __device__ __forceinline__ void tile_adj_step2(const TileArgs &a, float2 *G, int
             v[p1] = col[p1 * TB];
             col[p1 * TB] = make_float2(0.f, 0.f);
         }
-        dif_network<4, true>(v);
+        dif_network<4, true, true>(v);
         float2 *p = Xc + (long long)j * a.nbins + (n2 + a.cq) * sl;
         const int hi = live ? a.nq - a.cq - n2 : 0;
         const int lo = live ? T::NOS - a.cq - n2 : T::NOS;

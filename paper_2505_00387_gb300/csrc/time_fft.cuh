@@ -109,7 +109,7 @@ template <class F, bool INV>
 __device__ __forceinline__ void frame_fft(float2 *v, float2 *sm, const FrameTwiddle &ft,
                                           const float2 *s_tw, int t) {
     constexpr int C = F::C;
-    dif_network<4, INV>(v);
+    dif_network<4, INV, true>(v);
     {
         float2 w[16];
 #pragma unroll
@@ -131,7 +131,7 @@ __device__ __forceinline__ void frame_fft(float2 *v, float2 *sm, const FrameTwid
     float2 *grp = sm + (t / C) * F::GS;
 #pragma unroll
     for (int b = 0; b < 16; ++b) v[b] = grp[C * b + c];
-    dif_network<4, INV>(v);
+    dif_network<4, INV, true>(v);
 #pragma unroll
     for (int m = 1; m < 16; ++m) {
         float2 w = s_tw[rev_bits_c<4>(m) * C + c];
@@ -154,16 +154,16 @@ __device__ __forceinline__ void frame_fft(float2 *v, float2 *sm, const FrameTwid
             const float2 x = grp[p1 * C + (n ^ p1)], y = grp[p1 * C + ((n + 16) ^ p1)];
             float2 w = s_tw[n * C + 16];               // exp(-2 pi i n / 32)
             if (INV) w.y = -w.y;
-            v[n] = odd ? cmul(csub(x, y), w) : cadd(x, y);
+            v[n] = odd ? cmul(csub2(x, y), w) : cadd2(x, y);
         }
-        dif_network<4, INV>(v);
+        dif_network<4, INV, true>(v);
     } else {
 #pragma unroll
         for (int j = 0; j < 16 / C; ++j) {
             const int p1 = c + C * j;
 #pragma unroll
             for (int i = 0; i < C; ++i) v[j * C + i] = grp[p1 * C + (i ^ (p1 & (C - 1)))];
-            dif_network<F::LC, INV>(v + j * C);
+            dif_network<F::LC, INV, true>(v + j * C);
         }
     }
 }
