@@ -178,11 +178,22 @@ __device__ __forceinline__ void store_gathers(float2 *row, int g, int G, int wid
 // TMEM (two accumulator buffers of 256 columns) and its lane 0 issues the MMAs;
 // warps 5..20 build the operand tiles into a ring of two shared-memory stages.
 // The producers pace the kernel (instructions, and latency of the operand
-// loads), so there are as many as 96 registers a thread allow, and with 64
-// gathers each thread's share of a K chunk is whole: one A and one B unit
-// (forward), two and one (adjoint).  The B operands of a chunk, and the
-// adjoint's trace, are loaded before the wait for a free stage.  Four kinds of mbarrier hand the stages and accumulators
-// around:
+// loads), so there are 16 warps of them: 21 warps in all leave 80 registers a
+// thread (six warps on one scheduler), which the adjoint keeps without spills
+// and the forward with two words.  A thread's share of a K chunk is one A and
+// one B unit (forward), one A unit an M tile and one B unit (adjoint).  A warp
+// whose A rows are all past the tile's traces, or past the curvatures, writes
+// none: the accumulator rows they would give are never read.  With fewer than
+// 64 gathers only the first 8 Gp threads have a B unit, and the others branch
+// around its loads (predicated off they still issue).
+// The B operands of a chunk are loaded before the wait for a free stage; the
+// adjoint's trace record too, or with fewer than 64 gathers (whose chunks are
+// short) a chunk ahead.  us a launch, 100 curvatures x 36 azimuths, 2000
+// traces, 256 samples, forward / adjoint: with 11 producer warps, these without
+// the three rules, with them: 4 gathers 554 / 585, 545 / 678, 456 / 612; 24
+// gathers 747 / 789, 608 / 701, 554 / 646; 64 gathers 1259 / 1267, 725 / 835,
+// 680 / 828 (where the branch and the early record would cost 2 %).
+// Four kinds of mbarrier hand the stages and accumulators around:
 //   full[s]   producers -> MMA    (stage s written; one arrival per producer thread)
 //   empty[s]  MMA -> producers    (tcgen05.commit: the MMAs reading stage s are done)
 //   accf[b]   MMA -> epilogue     (tcgen05.commit after an item's last chunk)
@@ -238,6 +249,7 @@ __device__ __forceinline__ bool tc_wait_bar(const TcArgs &a, uint64_t *bar, uint
 // ------------------------------------------------------------- forward
 // Item = (bin k, row tile of <= 128 traces of slice j); K chunks of 32 q
 // samples (64 interleaved bf16 K-elements); accumulator 128 x 4Gp.
+template <bool WHOLE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__restrict__ Y) {
     extern __shared__ unsigned char smem_raw[];
@@ -325,25 +337,28 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
                 ka = (unsigned long long)k * tr->A;
                 kb = (unsigned long long)k * tr->B;
             }
-            const float2 st8 = cis_fixed(kb, -1.f);
+            float2 st8 = make_float2(1.f, 0.f);
+            if (trace) st8 = cis_fixed(kb, -1.f);
             // B unit: slice sl, gather g, 8 q samples
             const int rest = tc_div(pid, Gp, inv_gp);
             const int g = pid - rest * Gp, sl = rest & 1, lbb = rest >> 1;
-            const bool col = pid < 8 * Gp;
+            const bool col = WHOLE || pid < 8 * Gp;
             const float2 *Xs = (sl ? Xn : Xj) + g;
             for (int c = 0; c < nch; ++c, ++cc) {
                 float2 x[8];
+                if (col) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int l = 32 * c + 8 * lbb + i;
-                    x[i] = make_float2(0.f, 0.f);
-                    if (col && l < a.nq && g < a.G) x[i] = __ldg(Xs + (long long)l * a.G);
+                    for (int i = 0; i < 8; ++i) {
+                        const int l = 32 * c + 8 * lbb + i;
+                        x[i] = make_float2(0.f, 0.f);
+                        if (l < a.nq && g < a.G) x[i] = __ldg(Xs + (long long)l * a.G);
+                    }
                 }
                 const int st = cc & 1;
                 if (!tc_wait_bar(a, &bars.empty[st], ((cc >> 1) & 1) ^ 1, abort)) break;
                 unsigned char *ahi = sm + st * stage_bytes, *alo = ahi + kTileA;
                 unsigned char *bhi = alo + kTileA, *blo = bhi + bbytes;
-                {
+                if (t0 + 8 * (pid >> 5) < t1) {      // a warp holds 8 traces
                     // A: E[h][l] for 128 traces x 32 q samples, (Re, Im) interleaved
                     float2 e[8];
                     if (trace) {
@@ -437,6 +452,7 @@ slice_fwd_tc_kernel(const TcArgs a, const float2 *__restrict__ X, float2 *__rest
 // Item = (bin k, slice j); M = q (nmt tiles of 128), K = the traces of
 // slices j (weight w0) and j - 1 (weight w1) in chunks of 32; accumulator
 // nmt x (128 x 2Gp).
+template <bool WHOLE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__restrict__ Xh) {
     extern __shared__ unsigned char smem_raw[];
@@ -531,25 +547,34 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
             const int hh = pid & 31;
             const int tq = tc_div(pid, Gp, inv_gp);
             const int g = pid - tq * Gp;
-            const bool col = pid < 8 * Gp;
+            const bool col = WHOLE || pid < 8 * Gp;
+            unsigned long long rA = 0, rB = 0;
+            float rw = 0.f;
+            auto record = [&](int p) {           // of trace p of the two slices
+                if (p >= ntot) return;
+                const TraceGeo *tr = a.geo + (p < n1 ? a0 + p : b0 + (p - n1));
+                rA = tr->A;
+                rB = tr->B;
+                rw = p < n1 ? tr->w0 : tr->w1;
+            };
+            if (!WHOLE) record(hh);
             for (int c = 0; c < nch; ++c, ++cc) {
                 const int p = 32 * c + hh;
-                unsigned long long ka = 0, kb = 0;
-                float wgt = 0.f;
-                if (p < ntot) {
-                    const TraceGeo tr = a.geo[p < n1 ? a0 + p : b0 + (p - n1)];
-                    ka = (unsigned long long)k * tr.A;
-                    kb = (unsigned long long)k * tr.B;
-                    wgt = p < n1 ? tr.w0 : tr.w1;
-                }
+                if (WHOLE) record(p);
+                const unsigned long long ka = (unsigned long long)k * rA;
+                const unsigned long long kb = (unsigned long long)k * rB;
+                const float wgt = rw;
+                if (!WHOLE) record(p + 32);
                 float2 y[4];
+                if (col) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int py = 32 * c + 4 * tq + i;
-                    y[i] = make_float2(0.f, 0.f);
-                    if (col && py < ntot && g < a.G)
-                        y[i] = __ldg(py < n1 ? Ya + (long long)py * a.G + g
-                                             : Yb + (long long)(py - n1) * a.G + g);
+                    for (int i = 0; i < 4; ++i) {
+                        const int py = 32 * c + 4 * tq + i;
+                        y[i] = make_float2(0.f, 0.f);
+                        if (py < ntot && g < a.G)
+                            y[i] = __ldg(py < n1 ? Ya + (long long)py * a.G + g
+                                                 : Yb + (long long)(py - n1) * a.G + g);
+                    }
                 }
                 const int st = cc & 1;
                 if (!tc_wait_bar(a, &bars.empty[st], ((cc >> 1) & 1) ^ 1, abort)) break;
@@ -558,7 +583,8 @@ slice_adj_tc_kernel(const TcArgs a, const float2 *__restrict__ Yh, float2 *__res
                 const float2 st8 = cis_fixed(kb, 1.f);
                 for (int mt = 0; mt < nmt; ++mt) {
                     // A: w conj(E)[l][h], rows l of the M tile, K = 32 traces
-                    const int lr = 8 * (pid >> 5), l0 = 128 * mt + lr;
+                    const int lr = 8 * (pid >> 5), l0 = 128 * mt + lr;   // a warp's 8 rows
+                    if (l0 >= a.nq) break;
                     unsigned char *ahi = st0 + (2 * mt) * kTileA, *alo = ahi + kTileA;
                     float2 e[8];
                     if (p < ntot) {
@@ -680,8 +706,11 @@ cudaError_t configure_tc_kernels(Plan &p, int num_sms, int max_smem) {
     const size_t sf = tc_smem_bytes(p.tc_gp, false), sa = tc_smem_bytes(p.tc_gp, true);
     if ((int)sf > max_smem || (int)sa > max_smem) return cudaErrorInvalidConfiguration;
     cudaError_t e;
-    if ((e = raise_smem_limit(slice_fwd_tc_kernel, max_smem))) return e;
-    if ((e = raise_smem_limit(slice_adj_tc_kernel, max_smem))) return e;
+    if ((e = raise_smem_limit(slice_fwd_tc_kernel<false>, max_smem)) ||
+        (e = raise_smem_limit(slice_fwd_tc_kernel<true>, max_smem)) ||
+        (e = raise_smem_limit(slice_adj_tc_kernel<false>, max_smem)) ||
+        (e = raise_smem_limit(slice_adj_tc_kernel<true>, max_smem)))
+        return e;
     p.smem_sfwd = sf;
     p.smem_sadj = sa;
     const long long items_f = (long long)p.nbins * p.tc_ntiles;
@@ -695,10 +724,11 @@ cudaError_t launch_slice_tc(Plan &p, bool adjoint, const float2 *in, float2 *out
                             cudaStream_t st, int *counter) {
     TcArgs a = tc_args(p, adjoint, counter);
     a.wide = p.ngather % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 31) == 0;
-    if (adjoint)
-        slice_adj_tc_kernel<<<p.slice_grid_adj, kTcThreads, p.smem_sadj, st>>>(a, in, out);
-    else
-        slice_fwd_tc_kernel<<<p.slice_grid_fwd, kTcThreads, p.smem_sfwd, st>>>(a, in, out);
+    const bool whole = 8 * a.Gp == kTcProdThreads;       // every producer has a B unit
+    auto *fwd = whole ? slice_fwd_tc_kernel<true> : slice_fwd_tc_kernel<false>;
+    auto *adj = whole ? slice_adj_tc_kernel<true> : slice_adj_tc_kernel<false>;
+    if (adjoint) adj<<<p.slice_grid_adj, kTcThreads, p.smem_sadj, st>>>(a, in, out);
+    else fwd<<<p.slice_grid_fwd, kTcThreads, p.smem_sfwd, st>>>(a, in, out);
     return cudaGetLastError();
 }
 
