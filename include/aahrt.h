@@ -246,7 +246,8 @@ int aahrt_adjoint(aahrt_plan *plan, const float *d, float *m, void *stream);
  * Plans of AAHRT_PRECISION_SPLIT_BF16 keep their spectra slice-major with
  * the gathers fastest: X[theta][k][q][g] and Y[j][k][i][g], where block j
  * holds the traces whose first azimuth slice is j (i = rank of the trace
- * among them, in input order). */
+ * among them, in input order).  A stage may use the plan's workspace, as the
+ * operators do: one call at a time on a plan. */
 int aahrt_apply_stage(aahrt_plan *plan, int stage, const void *in, void *out,
                       void *stream);
 
@@ -457,6 +458,12 @@ int aahrt_plan_test_stall(aahrt_plan *plan, int on);
  * kernels before it already queued (a solve already captured in the plan's
  * graph is not affected).  Not for production use. */
 int aahrt_plan_test_fail_adjoint(aahrt_plan *plan, int on);
+
+/* Test hook: while on, stages 0, 2, 3 and 5 of aahrt_apply_stage run the
+ * register-FFT kernels of the plan's operators (through a transposition of the
+ * spectrum) instead of the ones for natural-order spectra.  Plans whose stages
+ * run their operators' kernels anyway get AAHRT_ERR_UNSUPPORTED. */
+int aahrt_plan_test_stage_frames(aahrt_plan *plan, int on);
 
 const char *aahrt_status_string(int status);
 const char *aahrt_last_error(void);

@@ -102,6 +102,7 @@ _SIGS = {
     "aahrt_forward_noalloc": (c_int, [c_void_p, c_void_p, c_void_p, c_void_p]),
     "aahrt_plan_test_stall": (c_int, [c_void_p, c_int]),
     "aahrt_plan_test_fail_adjoint": (c_int, [c_void_p, c_int]),
+    "aahrt_plan_test_stage_frames": (c_int, [c_void_p, c_int]),
     "aahrt_q_axis_slowness": (c_int, [c_double, c_double, c_int, POINTER(c_double)]),
     "aahrt_nq_required": (c_int, [c_double, c_double, c_double, POINTER(c_int)]),
     "aahrt_partial_nmo": (c_int, [c_void_p, c_void_p, c_void_p, c_double, c_int, c_void_p]),
@@ -220,6 +221,10 @@ def aahrt_plan_test_stall(h, on: bool):
 
 def aahrt_plan_test_fail_adjoint(h, on: bool):
     check(load().aahrt_plan_test_fail_adjoint(h, int(bool(on))), "aahrt_plan_test_fail_adjoint")
+
+
+def aahrt_plan_test_stage_frames(h, on: bool):
+    check(load().aahrt_plan_test_stage_frames(h, int(bool(on))), "aahrt_plan_test_stage_frames")
 
 
 def aahrt_q_axis_slowness(pmin: float, pmax: float, nq: int):

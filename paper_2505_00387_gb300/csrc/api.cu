@@ -215,6 +215,42 @@ static cudaError_t reblock(Plan &p, bool model_side, const float *src, float *ds
     return cudaGetLastError();
 }
 
+// A stage of a bins-fastest plan on the natural-order spectra of the C ABI, by
+// the operators' own kernels on the workspace and a transposition on either
+// side: the slice steps (stages 1 and 4; the input's transposition also finds
+// the adjoint's bound), and under a test hook the time stages, which otherwise
+// run the shared-memory FFT kernels on natural spectra (a transposition of a
+// spectrum that fits L2 costs more than they do: stage 0 of 16 cubes 335 us
+// against 389).  us a call, bin-per-block kernels on natural spectra -> these,
+// stages 1 and 4: a 32 q x 8 azimuths cube 15 / 23 -> 20 / 20 (two launches
+// more), a 2000-trace gather 98 / 186 -> 103 / 123, 16 cubes of 200-3000 traces
+// 773 / 1172 -> 650 / 823, 8000 traces on 512 grid points 918 / 1674 -> 815 / 975.
+static cudaError_t stage_own_layout(Plan &p, int stage, const void *in, void *out,
+                                    cudaStream_t st) {
+    const float *fi = static_cast<const float *>(in);
+    const float2 *ci = static_cast<const float2 *>(in);
+    float *fo = static_cast<float *>(out);
+    float2 *co = static_cast<float2 *>(out);
+    const bool model = stage == 0 || stage == 1 || stage == 5;   // the spectrum moved first is X
+    float2 *spec = model ? p.X : p.Y, *other = model ? p.Y : p.X;
+    cudaError_t e;
+    switch (stage) {
+        case 0:
+        case 3:
+            if ((e = launch_r2c(p, model, fi, spec, st, false, false, false))) return e;
+            return launch_transpose_spec(p, model, spec, co, false, false, st);
+        case 1:
+        case 4:
+            if ((e = launch_transpose_spec(p, model, ci, spec, true, stage == 4, st)) ||
+                (e = launch_slice(p, stage == 4, spec, other, st)))
+                return e;
+            return launch_transpose_spec(p, !model, other, co, false, false, st);
+        default:
+            if ((e = launch_transpose_spec(p, model, ci, spec, true, false, st))) return e;
+            return launch_c2r(p, model, spec, fo, EPI_STORE, nullptr, FistaArgs{}, st);
+    }
+}
+
 int check_dev_ptr(const void *ptr, const char *name) {
     if (!ptr) return set_error(AAHRT_ERR_INVALID_ARG, "%s is NULL", name);
     if (reinterpret_cast<uintptr_t>(ptr) & 15)
@@ -749,32 +785,26 @@ int aahrt_apply_stage(aahrt_plan *plan, int stage, const void *in, void *out, vo
     const float2 *ci = static_cast<const float2 *>(in);
     float *fo = static_cast<float *>(out);
     float2 *co = static_cast<float2 *>(out);
+    if (stage < 0 || stage > 5)
+        return set_error(AAHRT_ERR_INVALID_ARG, "stage must be 0..5");
+    if (p.bins_fastest && (stage == 1 || stage == 4 || p.stage_frames)) {
+        e = stage_own_layout(p, stage, in, out, st);
+        return e ? cuda_fail(e, "stage launch") : AAHRT_OK;
+    }
     switch (stage) {
-        case 0: e = launch_r2c(p, true, fi, co, st, false, true); break;
+        case 0: e = launch_r2c(p, true, fi, co, st, false, true, false); break;
+        case 1: e = launch_slice(p, false, ci, co, st); break;
         case 2:
             e = launch_c2r(p, false, ci, fo, EPI_STORE, nullptr, FistaArgs{}, st, false, true);
             break;
-        case 3: e = launch_r2c(p, false, fi, co, st, false, true); break;
-        case 1:
-        case 4: {
-            const bool adj = stage == 4;
-            e = adj ? launch_ybound(p, ci, st) : cudaSuccess;
-            if (e) break;
-            if (!p.bins_fastest) {
-                e = launch_slice(p, adj, ci, co, st);
-                break;
-            }
-            // through the workspace, which holds the plan's own layout
-            float2 *src = adj ? p.Y : p.X, *dst = adj ? p.X : p.Y;
-            e = launch_transpose_spec(p, !adj, ci, src, true, st);
-            if (!e) e = launch_slice(p, adj, src, dst, st);
-            if (!e) e = launch_transpose_spec(p, adj, dst, co, false, st);
+        case 3: e = launch_r2c(p, false, fi, co, st, false, true, false); break;
+        case 4:
+            e = launch_ybound(p, ci, st);
+            if (!e) e = launch_slice(p, true, ci, co, st);
             break;
-        }
-        case 5:
+        default:
             e = launch_c2r(p, true, ci, fo, EPI_STORE, nullptr, FistaArgs{}, st, false, true);
             break;
-        default: return set_error(AAHRT_ERR_INVALID_ARG, "stage must be 0..5");
     }
     return e ? cuda_fail(e, "stage launch") : AAHRT_OK;
 }
@@ -892,6 +922,15 @@ int aahrt_plan_test_fail_adjoint(aahrt_plan *plan, int on) {
     if (!plan) return set_error(AAHRT_ERR_INVALID_ARG, "plan is NULL");
     if (on != 0 && on != 1) return set_error(AAHRT_ERR_INVALID_ARG, "on must be 0 or 1");
     plan->p->fail_adj = on != 0;
+    return AAHRT_OK;
+}
+
+int aahrt_plan_test_stage_frames(aahrt_plan *plan, int on) {
+    if (!plan) return set_error(AAHRT_ERR_INVALID_ARG, "plan is NULL");
+    if (on != 0 && on != 1) return set_error(AAHRT_ERR_INVALID_ARG, "on must be 0 or 1");
+    if (!plan->p->bins_fastest)
+        return set_error(AAHRT_ERR_UNSUPPORTED, "the plan's stages run its operators' kernels");
+    plan->p->stage_frames = on != 0;
     return AAHRT_OK;
 }
 

@@ -225,6 +225,7 @@ struct Plan {
     int tc_gp = 0;                 // gathers padded to a multiple of 8
     int4 *tc_tiles = nullptr;      // forward row tiles {slice, first, end, 0}
     bool fail_adj = false;         // test hook: slice adjoints report a failed launch
+    bool stage_frames = false;     // test hook: stages 0, 2, 3, 5 on the operators' kernels
     bool tc_stall = false;         // test hook: tensor-core kernels issue no MMAs
     int tc_ntiles = 0;
     // deconvolutive operator: wavelet convolved with every trace in time
@@ -266,9 +267,11 @@ int set_error(int code, const char *fmt, ...);
 int cuda_fail(cudaError_t e, const char *what);
 
 // stage launchers (stream-ordered, no synchronisation); `natural`: the
-// spectrum is X[bin][q][theta] / Y[bin][trace] whatever the plan's layout
+// spectrum is X[bin][q][theta] / Y[bin][trace] whatever the plan's layout;
+// bound: raise the plan's spectrum bound table (data side)
 cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
-                       cudaStream_t st, bool blocked = false, bool natural = false);
+                       cudaStream_t st, bool blocked = false, bool natural = false,
+                       bool bound = true);
 cudaError_t launch_c2r(Plan &p, bool model_side, const float2 *in, float *out,
                        int epi, const float *aux, FistaArgs fa, cudaStream_t st,
                        bool blocked = false, bool natural = false);
@@ -288,9 +291,10 @@ cudaError_t configure_gather_frames(Plan &p, int max_smem);
 cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *in, void *out,
                          const float *aux, const FistaArgs &fa, bool blocked, bool bound,
                          cudaStream_t st);
-// a spectrum between its natural and its bins-fastest layout (every cube)
+// a spectrum between its natural and its bins-fastest layout (every cube);
+// bound (data spectra to bins): raise the plan's spectrum bound table
 cudaError_t launch_transpose_spec(Plan &p, bool model_side, const float2 *in, float2 *out,
-                                  bool to_bins, cudaStream_t st);
+                                  bool to_bins, bool bound, cudaStream_t st);
 // fused synthesis + analysis of one FISTA half-iteration (column-blocked state)
 cudaError_t launch_c2r_r2c(Plan &p, bool model_side, float2 *spec, const float *aux,
                            FistaArgs fa, cudaStream_t st);

@@ -399,10 +399,7 @@ cudaError_t ybound_begin(Plan &p, cudaStream_t st) {
 
 cudaError_t launch_ybound(Plan &p, const float2 *Y, cudaStream_t st) {
     if (!p.ymax || p.precision == 1 || p.slice_interp == AAHRT_SLICE_DIRECT) return cudaSuccess;
-    cudaError_t e = p.bins_fastest
-                        ? ybound_begin(p, st)
-                        : cudaMemsetAsync(p.ymax, 0,
-                                          (size_t)p.ncube * p.nychunk * sizeof(unsigned), st);
+    cudaError_t e = cudaMemsetAsync(p.ymax, 0, (size_t)p.ncube * p.nychunk * sizeof(unsigned), st);
     if (e) return e;
     ybound_kernel<<<dim3(p.ngroups_total, p.nychunk), 256, 0, st>>>(
         p.groups, Y, p.nbins, p.ychunk_log, p.nychunk, p.ymax);

@@ -58,36 +58,73 @@ cudaError_t configure_tile_kernels(Plan &p, int num_sms, int max_smem) {
     return cudaSuccess;
 }
 
-// One cube's block of [rows][cols] -> [cols][rows], 32 x 32 tiles.
-__global__ void transpose_kernel(const float2 *__restrict__ in, float2 *__restrict__ out,
-                                 const SpecBlock *__restrict__ blk, int nbins, int to_bins) {
-    __shared__ float2 s[32][33];
+// One cube's block of [rows][cols] -> [cols][rows], in tiles of 32 x 64 (64 x 64:
+// 4 % more of a stage).  BOUND (rows = bins): also the largest |re| + |im| of
+// each chunk of bins (of 64 or more, so a tile lies in one) into the cube's row
+// of the bound table, where a pass of its own over the spectrum per azimuth
+// group took a third of stage 4.
+constexpr int kRows = 32;
+template <bool BOUND>
+__global__ void __launch_bounds__(256)
+transpose_kernel(const float2 *__restrict__ in, float2 *__restrict__ out,
+                 const SpecBlock *__restrict__ blk, int nbins, int to_bins, unsigned *ymax,
+                 int nychunk, int ychunk_log) {
+    __shared__ float2 s[kRows][65];
+    __shared__ unsigned s_max;
     const SpecBlock b = blk[blockIdx.z];
     const int rows = to_bins ? nbins : b.ncol, cols = to_bins ? b.ncol : nbins;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int r0 = blockIdx.y * 32; r0 < rows; r0 += gridDim.y * 32)
-        for (int c0 = blockIdx.x * 32; c0 < cols; c0 += gridDim.x * 32) {
-            for (int i = ty; i < 32; i += 8)
-                if (r0 + i < rows && c0 + tx < cols)
-                    s[i][tx] = in[b.off + (long long)(r0 + i) * cols + c0 + tx];
-            __syncthreads();
-            for (int i = ty; i < 32; i += 8)
-                if (c0 + i < cols && r0 + tx < rows)
-                    out[b.off + (long long)(c0 + i) * rows + r0 + tx] = s[tx][i];
-            __syncthreads();
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int ox = threadIdx.x % kRows, oy = threadIdx.x / kRows;
+    const int c0 = blockIdx.x * 64;
+    if (c0 >= cols) return;              // (a cube of fewer columns than the largest)
+    for (int r0 = blockIdx.y * kRows; r0 < rows; r0 += gridDim.y * kRows) {
+        float2 v[kRows / 4];
+#pragma unroll
+        for (int i = 0; i < kRows / 4; ++i) {
+            v[i] = make_float2(0.f, 0.f);
+            if (r0 + ty + 4 * i < rows && c0 + tx < cols)
+                v[i] = __ldcs(in + b.off + (long long)(r0 + ty + 4 * i) * cols + c0 + tx);
         }
+        if (BOUND && threadIdx.x == 0) s_max = 0u;
+        float m = 0.f;
+#pragma unroll
+        for (int i = 0; i < kRows / 4; ++i) {
+            s[ty + 4 * i][tx] = v[i];
+            m = fmaxf(m, fabsf(v[i].x) + fabsf(v[i].y));
+        }
+        __syncthreads();
+        if (BOUND) {
+            const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+            if ((threadIdx.x & 31) == 0 && w > 0u) atomicMax(&s_max, w);
+        }
+#pragma unroll
+        for (int i = 0; i < kRows / 4; ++i) {
+            const int c = oy + i * (256 / kRows);
+            if (c0 + c < cols && r0 + ox < rows)
+                out[b.off + (long long)(c0 + c) * rows + r0 + ox] = s[ox][c];
+        }
+        __syncthreads();
+        if (BOUND && threadIdx.x == 0) {
+            unsigned *e = ymax + (long long)blockIdx.z * nychunk + (r0 >> ychunk_log);
+            if (s_max > *(volatile unsigned *)e) atomicMax(e, s_max);
+        }
+    }
 }
 
 cudaError_t launch_transpose_spec(Plan &p, bool model_side, const float2 *in, float2 *out,
-                                  bool to_bins, cudaStream_t st) {
+                                  bool to_bins, bool bound, cudaStream_t st) {
+    cudaError_t e;
+    if (bound && (e = ybound_begin(p, st))) return e;
     const SpecBlock *blk = model_side ? p.spec_model : p.spec_data;
     const int ncol = model_side ? (int)p.cols_model : p.max_ntr;
-    const int gr = ((to_bins ? p.nbins : ncol) + 31) / 32, gc = ((to_bins ? ncol : p.nbins) + 31) / 32;
-    for (int c0 = 0; c0 < p.ncube; c0 += 65535) {
-        const int n = std::min(p.ncube - c0, 65535);
-        transpose_kernel<<<dim3(gc, std::min(gr, 65535), n), 256, 0, st>>>(in, out, blk + c0, p.nbins,
-                                                                          to_bins ? 1 : 0);
-    }
+    const int rows = to_bins ? p.nbins : ncol, cols = to_bins ? ncol : p.nbins;
+    auto *kern = bound ? transpose_kernel<true> : transpose_kernel<false>;
+    for (int c0 = 0; c0 < p.ncube; c0 += 65535)
+        kern<<<dim3((cols + 63) / 64, std::min((rows + kRows - 1) / kRows, 65535),
+                    std::min(p.ncube - c0, 65535)), 256, 0, st>>>(
+            in, out, blk + c0, p.nbins, to_bins ? 1 : 0, p.ymax + (long long)c0 * p.nychunk,
+            p.nychunk, p.ychunk_log);
+    p.launches[6]++;
     return cudaGetLastError();
 }
 

@@ -1,8 +1,8 @@
 // Time-axis stages of the AAHRT (Algorithms 1 and 2, steps 1-2 and 4-5) on
-// spectra whose columns or gathers are fastest: every plan's stages on natural
-// layouts (aahrt_apply_stage, the pull scan), the solvers' half-iterations of
-// gathers-fastest plans, and the operators of the plans the register-FFT
-// kernels (time_fft.cuh) do not serve:
+// spectra whose columns or gathers are fastest: the pull scan of every plan,
+// stages 0, 2, 3 and 5 of aahrt_apply_stage on FP32 plans, the solvers'
+// half-iterations of gathers-fastest plans, and the operators of the plans the
+// register-FFT kernels (time_fft.cuh) do not serve:
 //
 //   r2c: X[k][c] = sum_n (G in)[n][c] exp(-2 pi i k n / Nfft), k < nbins
 //        where G resamples each column: the time stretch S (model side,
@@ -528,7 +528,7 @@ static void c2r_launch(bool model_side, int grid, size_t smem, cudaStream_t st,
     else { constexpr int IPc = AAHRT_INTERP_KEYS; STMT; }
 
 cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
-                       cudaStream_t st, bool blocked, bool natural) {
+                       cudaStream_t st, bool blocked, bool natural, bool bound) {
     const ColGroup *cg = model_side ? (blocked ? p.cg_model_blk : p.cg_model)
                                     : (blocked ? p.cg_data_blk : p.cg_data);
     const int n = model_side ? p.ncg_model : p.ncg_data;
@@ -537,16 +537,14 @@ cudaError_t launch_r2c(Plan &p, bool model_side, const float *in, float2 *out,
     const size_t smem = model_side ? p.smem_r2c_model : p.smem_r2c_data;
     const int stage = model_side ? 0 : 3;
     YBound yb{};
-    // (natural spectra of bins-fastest plans: aahrt_apply_stage computes the
-    // bound from the spectrum it is given)
-    if (!model_side && !(p.bins_fastest && natural)) {
+    if (!model_side && bound) {
         const cudaError_t e = p.bins_fastest ? ybound_begin(p, st) : ybound_reset(p, st, &yb);
         if (e) return e;
     }
     prof_begin(p, stage, st);
     if (p.gather_frames ? !blocked : p.bins_fastest && !natural) {
         const cudaError_t e = launch_frame(p, 0, model_side, EPI_STORE, in, out, nullptr,
-                                           FistaArgs{}, blocked, !model_side, st);
+                                           FistaArgs{}, blocked, !model_side && bound, st);
         prof_end(p, st);
         p.launches[stage]++;
         return e;
