@@ -465,6 +465,12 @@ int aahrt_plan_test_fail_adjoint(aahrt_plan *plan, int on);
  * run their operators' kernels anyway get AAHRT_ERR_UNSUPPORTED. */
 int aahrt_plan_test_stage_frames(aahrt_plan *plan, int on);
 
+/* For tests: the shape of the plan's register-FFT blocks: column pairs a block
+ * holds, and pairs an analysis block of one pair takes in turn (model and data
+ * columns); zeros where the plan does not use these kernels. */
+int aahrt_plan_test_frame_shape(const aahrt_plan *plan, int *pairs, int *turn_model,
+                                int *turn_data);
+
 const char *aahrt_status_string(int status);
 const char *aahrt_last_error(void);
 

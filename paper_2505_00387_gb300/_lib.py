@@ -103,6 +103,8 @@ _SIGS = {
     "aahrt_plan_test_stall": (c_int, [c_void_p, c_int]),
     "aahrt_plan_test_fail_adjoint": (c_int, [c_void_p, c_int]),
     "aahrt_plan_test_stage_frames": (c_int, [c_void_p, c_int]),
+    "aahrt_plan_test_frame_shape": (c_int, [c_void_p, POINTER(c_int), POINTER(c_int),
+                                            POINTER(c_int)]),
     "aahrt_q_axis_slowness": (c_int, [c_double, c_double, c_int, POINTER(c_double)]),
     "aahrt_nq_required": (c_int, [c_double, c_double, c_double, POINTER(c_int)]),
     "aahrt_partial_nmo": (c_int, [c_void_p, c_void_p, c_void_p, c_double, c_int, c_void_p]),
@@ -225,6 +227,13 @@ def aahrt_plan_test_fail_adjoint(h, on: bool):
 
 def aahrt_plan_test_stage_frames(h, on: bool):
     check(load().aahrt_plan_test_stage_frames(h, int(bool(on))), "aahrt_plan_test_stage_frames")
+
+
+def aahrt_plan_test_frame_shape(h):
+    v = [c_int() for _ in range(3)]
+    check(load().aahrt_plan_test_frame_shape(h, *[ctypes.byref(x) for x in v]),
+          "aahrt_plan_test_frame_shape")
+    return tuple(x.value for x in v)
 
 
 def aahrt_q_axis_slowness(pmin: float, pmax: float, nq: int):

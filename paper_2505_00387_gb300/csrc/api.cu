@@ -934,6 +934,17 @@ int aahrt_plan_test_stage_frames(aahrt_plan *plan, int on) {
     return AAHRT_OK;
 }
 
+int aahrt_plan_test_frame_shape(const aahrt_plan *plan, int *pairs, int *turn_model,
+                                int *turn_data) {
+    if (!plan || !pairs || !turn_model || !turn_data)
+        return set_error(AAHRT_ERR_INVALID_ARG, "plan or an output is NULL");
+    const Plan &p = *plan->p;
+    *pairs = p.frame_pairs;
+    *turn_model = p.frame_pairs ? p.frame_seq_model : 0;
+    *turn_data = p.frame_pairs ? p.frame_seq_data : 0;
+    return AAHRT_OK;
+}
+
 const char *aahrt_status_string(int status) {
     switch (status) {
         case AAHRT_OK: return "success";
