@@ -148,7 +148,8 @@ struct Plan {
     TraceGeo *geo = nullptr;
     SliceGroup *groups = nullptr;
     int *slice_start = nullptr;    // per distinct geometry: first sorted trace of each slice
-    TraceGeo *geo_adj = nullptr;   // the same traces in the adjoint slice kernel's order
+    TraceGeo *geo_adj = nullptr;   // the same traces in the order of the bin-per-block
+                                   // adjoint (plans that run it, else null)
     // Amplitude bound of the data spectrum for the adjoint spread's
     // fixed-point scale: ymax[cube][chunk] = max |re| + |im| of Y over the
     // chunk's 2^ychunk_log bins (float bits; written by the data-side

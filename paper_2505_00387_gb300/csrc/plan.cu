@@ -120,11 +120,13 @@ static unsigned long long to_fixed64(double x) {
 
 struct CubeGeo {
     std::vector<TraceGeo> sorted;      // by slice, then r^2 (forward order)
-    std::vector<TraceGeo> sorted_adj;  // by slice, then trace index (adjoint order)
+    std::vector<TraceGeo> sorted_adj;  // by slice, then trace index (the order of the
+                                       // bin-per-block adjoint), where that runs
     std::vector<int> start;  // start[j]: first sorted trace with j0 == j (size ntheta+1)
 };
 
-static CubeGeo bin_cube(const Plan &p, const double *hx, const double *hy, int ntr) {
+static CubeGeo bin_cube(const Plan &p, const double *hx, const double *hy, int ntr,
+                        bool adj_order) {
     CubeGeo g;
     std::vector<TraceGeo> tr(ntr);
     const double dth = M_PI / p.ntheta;
@@ -172,6 +174,7 @@ static CubeGeo bin_cube(const Plan &p, const double *hx, const double *hy, int n
     for (int j = 0; j < p.ntheta; ++j) g.start[j + 1] += g.start[j];
     g.sorted.resize(ntr);
     for (int i = 0; i < ntr; ++i) g.sorted[i] = tr[idx[i]];
+    if (!adj_order) return g;
     std::vector<int> ida(ntr);
     std::iota(ida.begin(), ida.end(), 0);
     std::stable_sort(ida.begin(), ida.end(), [&](int a, int b) { return tr[a].j0 < tr[b].j0; });
@@ -501,7 +504,9 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
 
     // ------------------------------------------------ per-cube geometry
     std::vector<CubeGeo> cg(ndist);
-    for (int c = 0; c < ndist; ++c) cg[c] = bin_cube(*p, geoms[c].hx, geoms[c].hy, geoms[c].ntr);
+    const bool adj_order = !tc && !direct && !p->bins_fastest;
+    for (int c = 0; c < ndist; ++c)
+        cg[c] = bin_cube(*p, geoms[c].hx, geoms[c].hy, geoms[c].ntr, adj_order);
     std::vector<long long> geo_off(ndist, 0);
     std::vector<TraceGeo> geo_all, geo_adj_all;
     std::vector<int> ss_all;
