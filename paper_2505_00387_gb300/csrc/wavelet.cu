@@ -52,7 +52,8 @@ wavelet_kernel(const float *__restrict__ in, float *__restrict__ out,
 cudaError_t launch_wavelet(Plan &p, int mode, const float *in, float *out, const float *aux,
                            cudaStream_t st, bool blocked) {
     const ColGroup *groups = blocked ? p.cg_data_blk : p.cg_data;
-    const size_t smem = (size_t)(((p.nw + 3) & ~3) + p.nt * 2 * p.pairs) * sizeof(float);
+    const int cols = 2 << (blocked ? p.blk_lp : p.lp);           // of a group
+    const size_t smem = (size_t)(((p.nw + 3) & ~3) + p.nt * cols) * sizeof(float);
     const int grid = blocked ? p.ncg_data_blk : p.ncg_data;
     switch (mode) {
         case WAV_CONV:
