@@ -284,10 +284,10 @@ cudaError_t launch_slice_tiles(Plan &p, bool adjoint, const float2 *in, float2 *
 cudaError_t configure_tile_kernels(Plan &p, int num_sms, int max_smem);
 // the time stages of bins-fastest spectra (time_fft.cuh): op 0 analysis,
 // 1 synthesis, 2 both fused; bound: raise the plan's spectrum bound table
-bool frame_serves(int L, int nt, int ntau, int ns, int max_smem);
+bool frame_serves(int L, int nt, int ntau, int max_smem);
 cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem);
 // the same stages with the gathers fastest (tensor-core plans, row-major rows)
-bool gather_frames_serve(int L, int nt, int ntau, int ns, int max_smem);
+bool gather_frames_serve(int L, int nt, int ntau, int max_smem);
 cudaError_t configure_gather_frames(Plan &p, int max_smem);
 cudaError_t launch_frame(Plan &p, int op, bool model_side, int epi, const void *in, void *out,
                          const float *aux, const FistaArgs &fa, bool blocked, bool bound,

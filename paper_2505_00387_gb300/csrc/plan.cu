@@ -467,8 +467,8 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     // time, and 8-byte pieces at a column stride cost its forward more (314 ->
     // 361 us, 100 curvatures x 2000 traces) than the faster time stages gave.
     p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512 &&
-                      frame_serves(p->L, p->nt, p->ntau, p->ns, optin);
-    p->gather_frames = tc && gather_frames_serve(p->L, p->nt, p->ntau, p->ns, optin);
+                      frame_serves(p->L, p->nt, p->ntau, optin);
+    p->gather_frames = tc && gather_frames_serve(p->L, p->nt, p->ntau, optin);
     const size_t per_slice = (size_t)std::max(ld_interleaved(p->nos), ld_split(p->nos)) *
                              sizeof(float2);
     if (opts.theta_group > 0) {

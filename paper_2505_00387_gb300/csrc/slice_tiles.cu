@@ -19,8 +19,6 @@ static TileArgs tile_args(const Plan &p, int *counter) {
     a.total = (long long)p.ngroups_total * a.ntiles;
     a.nq = p.nq;
     a.ntheta = p.ntheta;
-    a.nos = p.nos;
-    a.Lq = p.Lq;
     a.cq = p.cq;
     a.scale = (float)(1.0 / p.nfft);
     a.phicap = (float)p.phicap;

@@ -44,7 +44,7 @@ struct TileArgs {
     const float2 *__restrict__ tw;
     int *counter;
     long long total;                       // groups x tiles
-    int nbins, ntiles, nq, ntheta, nos, Lq, cq;
+    int nbins, ntiles, nq, ntheta, cq;
     float scale;
     float phicap;                          // bound on one kernel weight
     unsigned *ymax;
@@ -156,7 +156,6 @@ __device__ __forceinline__ void tile_fwd_step2(float2 *G, const float2 *s_tw, in
 #pragma unroll
         for (int p0 = 0; p0 < 16; p0 += T::NSUB) {
             const int p1 = p0 + sub;
-            if (T::NSUB > 16 && p1 >= 16) break;
             float2 *col = G + p1 * TB + bin;
             float2 v[R];
 #pragma unroll
@@ -362,7 +361,6 @@ __device__ __forceinline__ void tile_adj_step1(float2 *G, int sub, int bin, cons
 #pragma unroll
         for (int p0 = 0; p0 < 16; p0 += T::NSUB) {
             const int p1 = p0 + sub;
-            if (T::NSUB > 16 && p1 >= 16) break;
             const PlanePair<TB> pl(reinterpret_cast<const int *>(G + p1 * TB) + bin);
             float2 v[R];
 #pragma unroll

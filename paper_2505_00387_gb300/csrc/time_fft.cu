@@ -33,7 +33,7 @@ static size_t frame_analysis_smem(int L, int seq, int nrows, int nfrac) {
 }
 
 // Shared memory of the largest time kernel of frames of 2^L samples.
-static size_t frame_plan_smem(int L, int pairs, int nt, int ntau, int ns) {
+static size_t frame_plan_smem(int L, int pairs, int nt, int ntau) {
     const int nrows = std::max(nt, ntau), nfrac = nt;
     switch (L) {
         case 9: return frame_most<2>(pairs, nrows, nfrac);
@@ -44,16 +44,16 @@ static size_t frame_plan_smem(int L, int pairs, int nt, int ntau, int ns) {
     }
 }
 
-bool frame_serves(int L, int nt, int ntau, int ns, int max_smem) {
+bool frame_serves(int L, int nt, int ntau, int max_smem) {
     // (1 KB stays for the kernels' static shared memory)
-    return L >= 9 && L <= 13 && frame_plan_smem(L, 1, nt, ntau, ns) + 1024 <= (size_t)max_smem;
+    return L >= 9 && L <= 13 && frame_plan_smem(L, 1, nt, ntau) + 1024 <= (size_t)max_smem;
 }
 
 static int gather_pairs(int L) { return L >= 12 ? 2 : 4096 >> L; }
 
-bool gather_frames_serve(int L, int nt, int ntau, int ns, int max_smem) {
+bool gather_frames_serve(int L, int nt, int ntau, int max_smem) {
     return L >= 9 && L <= 13 &&
-           frame_plan_smem(L, gather_pairs(L), nt, ntau, ns) + 1024 <= (size_t)max_smem;
+           frame_plan_smem(L, gather_pairs(L), nt, ntau) + 1024 <= (size_t)max_smem;
 }
 
 cudaError_t configure_gather_frames(Plan &p, int max_smem) {
@@ -74,7 +74,7 @@ cudaError_t configure_frame_kernels(Plan &p, int num_sms, int max_smem) {
     p.frame_pairs = std::max(1, 256 / (p.nfft / 16));
     while (p.frame_pairs > 1 &&
            (groups / p.frame_pairs < num_sms ||
-            frame_plan_smem(p.L, p.frame_pairs, p.nt, p.ntau, p.ns) + 1024 > (size_t)max_smem))
+            frame_plan_smem(p.L, p.frame_pairs, p.nt, p.ntau) + 1024 > (size_t)max_smem))
         p.frame_pairs /= 2;
     // pairs an analysis block of one pair takes in turn: as many as cost at most
     // 3 % more rounds of resident blocks than one at a time, within the shared
