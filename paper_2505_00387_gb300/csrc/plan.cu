@@ -237,8 +237,14 @@ static int validate_geom(const aahrt_geom *g, int idx, bool q_explicit) {
 // Bins per tile and azimuth slices per work item of the bins-fastest slice
 // kernels.  An item walks its nj slices and one more (the neighbour its first
 // or last interval shares), so its time goes as (nj + 1) x tile, and the items
-// run in ceil(items / resident blocks) rounds: the pair with the smallest
-// product, larger tiles (a whole warp on one trace) on a tie.
+// run in items / resident blocks rounds, and half a round more for the last
+// (0.25 to 1 choose alike): the pair with the smallest product.  16-bin tiles where both serve (up to 128 points) count
+// 1.4 times: every curvature row moves in 128-byte pieces and two traces share a
+// warp.  Forward + adjoint slice steps of 59 plans (9-64 curvatures, 2-72
+// azimuths, 60-5000 traces, 1-24 cubes), against a weight of 1.15: 0.97 to 1.37
+// times as fast, 1.03 on average; on 31 others, tried at every split, weights of
+// 1.0, 1.15 and 1.4 choose splits that take 1.20, 1.13 and 1.04 times the best
+// time (1.4 without the half round: 1.08).
 static void choose_tiles(Plan &p, bool group_fixed, int ncube, int sms) {
     const long long blocks = (long long)sms * 3;
     double best = 1e300;
@@ -250,7 +256,7 @@ static void choose_tiles(Plan &p, bool group_fixed, int ncube, int sms) {
             const long long groups = (p.ntheta + nj - 1) / nj;
             const long long items = groups * ((p.nbins + tile - 1) / tile) * ncube;
             const double rounds = items > blocks ? (double)items / blocks + 0.5 : 1.0;
-            const double cost = rounds * (nj + 1) * tile * (tile == 16 && p.nos <= 128 ? 1.15 : 1.0);
+            const double cost = rounds * (nj + 1) * tile * (tile == 16 && p.nos <= 128 ? 1.4 : 1.0);
             if (cost < best) {
                 best = cost;
                 p.tile = tile;
@@ -462,8 +468,13 @@ int build_plan(Plan **out, int ncube, int ndist, const aahrt_geom *geoms,
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
     // Bins fastest wherever its kernels exist: frames whose FFT registers hold
     // and q grids of two radix steps (32 points) up to two grids of 8 bins with
-    // three blocks an SM (512); measured on both sides in slice_tiles.cuh and
-    // time_fft.cuh.  The direct sum keeps natural spectra: it takes one bin at a
+    // three blocks an SM (512).  Whole operators at the edges, on natural
+    // spectra -> bins fastest, 12 azimuths x 400 samples, forward / adjoint us:
+    // 32 points, 5 taps, 60 traces 37 / 47 -> 23 / 31, 12 taps, 3000 traces
+    // 62 / 226 -> 43 / 80; 512 points 47 / 64 -> 40 / 47 and 70 / 266 -> 60 / 83;
+    // linear-k, 3000 traces 58 / 84 -> 34 / 60 (32) and 66 / 101 -> 52 / 64 (512);
+    // paper-scale axes cut to a few bins by fmax 62 / 92 -> 44 / 68; one azimuth
+    // of 4000 traces, the least gain, 91 / 207 -> 88 / 198.  The direct sum keeps natural spectra: it takes one bin at a
     // time, and 8-byte pieces at a column stride cost its forward more (314 ->
     // 361 us, 100 curvatures x 2000 traces) than the faster time stages gave.
     p->bins_fastest = !tc && !direct && p->nos >= 32 && p->nos <= 512 &&
