@@ -138,9 +138,9 @@ typedef struct {
                            Nfft = 8192, 1 beyond).  Plans whose time stages
                            hold the FFT in registers (Nfft 512..8192 with a
                            spreading kernel on 32..512 q points) use it for
-                           aahrt_apply_stage and the pull scan only,
-                           split-BF16 plans of those frames for these and the
-                           solvers */
+                           the time stages of aahrt_apply_stage and the pull
+                           scan only, split-BF16 plans of those frames for the
+                           solvers only */
     int autotune;       /* 1: pick spread_width, theta_group and time_pairs
                            at plan creation (see aahrt_plan_create); fields
                            set explicitly above are kept */

@@ -7,11 +7,12 @@
 // cube.  It keeps the q grids of two neighbouring slices in shared memory as
 // [grid point][bin], walks its slices in order, and in each interval
 // [theta_j, theta_j+1) handles the traces whose first slice is j.  A trace's
-// grid position differs from bin to bin, but a bin stays in its own bank, so
-// neither the forward's reads nor the adjoint's integer atomics conflict,
-// whatever the positions (with a bin per block and 32 traces per warp they
-// hit random banks: 3.7 wavefronts per atomic, measured).  Every global access
-// is a run of TB consecutive bins.
+// grid position differs from bin to bin, but a bin stays in its own bank, so in
+// tiles of 32 and 16 bins neither the forward's reads nor the adjoint's integer
+// atomics conflict, whatever the positions (with a bin per block and 32 traces
+// per warp they hit random banks: 3.7 wavefronts per atomic, measured); in
+// tiles of 8 bins (512-point grids) two of a warp's four traces do, half the
+// time.  Every global access is a run of TB consecutive bins.
 //
 // The nos-point DFT of a grid column stays inside the lanes of its bin:
 // nos = 16 R, n = n1 R + n2, p = p1 + 16 p2,
@@ -23,11 +24,11 @@
 //
 // Bound: issue (68-71 % of the slots) with the L1 / shared-memory pipe at
 // 57-71 %; the bin-per-block kernels had that pipe at 87-91 %, half of it
-// conflicts.  Per launch on 16 cubes of 200-3000 traces, 100 q x 36 azimuths,
-// 2048 bins (nos 256, W 7), bin per block -> these kernels: forward 823 -> 442
-// us, adjoint 1108 -> 622; one 2000-trace gather of the same axes 99 -> 72 and
-// 125 -> 92; one 8000-trace gather, 200 q x 72 azimuths (nos 512) 929 -> 593 and
-// 1400 -> 750.
+// conflicts.  Per launch on 16 cubes of 200-3000 traces, 64 q x 24 azimuths,
+// 2048 bins (nos 128, W 7), bin per block -> these kernels: forward 823 -> 440
+// us, adjoint 1108 -> 618; one 2000-trace gather, 100 q x 36 azimuths (nos 256,
+// W 6) 99 -> 71 and 125 -> 92; one 8000-trace gather, 200 q x 72 azimuths (nos
+// 512, W 6) 929 -> 595 and 1400 -> 756.
 #pragma once
 
 #include "fft.cuh"

@@ -4,7 +4,7 @@
 // Tiles of 32 bins where two grids of nos points leave room for three blocks
 // per SM (nos <= 128), of 16 bins for 256 points (and for small plans, whose
 // work items would not fill the SMs), of 8 for 512 points: half the traces of a
-// pair conflict then, but three blocks share an SM (594 / 765 us forward /
+// pair conflict then, but three blocks share an SM (595 / 756 us forward /
 // adjoint of the 8000-trace gather against 677 / 882 with 16 bins and one block
 // of 512 threads).
 #pragma once

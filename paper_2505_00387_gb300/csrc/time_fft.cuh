@@ -19,9 +19,9 @@
 // at 64 registers (four blocks of 256 threads an SM; 80 and three in the
 // analysis alone) instead of 128 and two.  Per launch on 16 cubes of 1001
 // samples and 200-3000 traces (4096-sample frames), shared-memory FFT ->
-// these kernels: data half 839 -> 443 us, model half 734 -> 481; analysis
-// 661 -> 429 (model) and 1064 -> 632 (data), synthesis 699 -> 468 (data) and
-// 977 -> 676 (model).
+// these kernels: data half 839 -> 442 us, model half 734 -> 477; of 32 such
+// cubes analysis 661 -> 431 (model) and 1064 -> 638 (data), synthesis 699 -> 469
+// (data) and 977 -> 685 (model).
 //
 // Shared-memory layout of an exchange: element (p0, i) of group p0 at
 // p0 (T + C) + i (the skew spreads the groups a half warp touches over the
@@ -46,7 +46,9 @@ struct Frame {
     static constexpr int THREADS = T > 256 ? T : 256;  // most threads of a block
     // blocks an SM holds: four (two of 512 threads) at 64 registers; the
     // analysis alone keeps 80, which its table entries and rows in flight need
-    // (430 against 535 us for the model columns of 32 cubes)
+    // (431 against 535 us for the model columns of 32 cubes; at 80 the model
+    // analyses of 2048 samples and fewer still spill 32 to 36 words, the other
+    // kernels 7 or fewer)
     static constexpr int MINB = T > 256 ? 2 : 4, MINB_ANA = T > 256 ? 1 : 3;
 };
 
